@@ -7,6 +7,7 @@
 #include <string>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "internal.h"
 
 namespace lqcd {
@@ -96,12 +97,7 @@ int lqcd_destroy(lqcd_ctx* ctx) {
   mrhs_release(ctx);
   force_release(ctx);
   traj_release(ctx);
-  if (ctx->gauge.owned) {
-    void* g[] = {ctx->gauge.u64, ctx->gauge.u32, ctx->gauge.u12, ctx->gauge.u8, ctx->gauge.u16,
-                 ctx->gauge.u32lo};
-    for (void* b : g)
-      if (b) cudaFree(b);
-  }
+  if (ctx->gauge.owned && ctx->gauge.block) cudaFree(ctx->gauge.block);
   for (auto& kv : ctx->batch_tables) cudaFree(kv.second);
   void* bufs[] = {ctx->partials, ctx->tickets, ctx->scalars, ctx->tmp_odd, ctx->bounds_word};
   for (void* b : bufs)
@@ -137,12 +133,7 @@ int lqcd_share_gauge(lqcd_ctx* ctx, const lqcd_ctx* src) {
   for (int d = 0; d < 4; ++d)
     if (ctx->dims[d] != src->dims[d]) return fail(ctx, LQCD_ERR_DIMS, "lqcd_share_gauge: lattices differ");
   if (!src->gauge.loaded) return fail(ctx, LQCD_ERR_STATE, "lqcd_share_gauge: source has no gauge field");
-  if (ctx->gauge.owned) {
-    void* g[] = {ctx->gauge.u64, ctx->gauge.u32, ctx->gauge.u12, ctx->gauge.u8, ctx->gauge.u16,
-                 ctx->gauge.u32lo};
-    for (void* b : g)
-      if (b) cudaFree(b);
-  }
+  if (ctx->gauge.owned && ctx->gauge.block) cudaFree(ctx->gauge.block);
   ctx->gauge = src->gauge;
   ctx->gauge.owned = false;
   free_workspace(ctx);  // captured graphs refer to the old link copies
@@ -157,18 +148,40 @@ int lqcd_set_gauge(lqcd_ctx* ctx, const double* U_dev) {
   GaugeCopies& gc = ctx->gauge;
   cudaError_t e;
   size_t vh = (size_t)ctx->Vh;
-  if (!gc.u64 && (e = cudaMalloc(&gc.u64, 2 * 4 * 9 * vh * sizeof(double2))) != cudaSuccess)
-    return cuda_check(ctx, e, "cudaMalloc(gauge fp64)");
-  if (!gc.u32 && (e = cudaMalloc(&gc.u32, 2 * 4 * 18 * vh * sizeof(float))) != cudaSuccess)
-    return cuda_check(ctx, e, "cudaMalloc(gauge fp32)");
-  if (!gc.u12 && (e = cudaMalloc(&gc.u12, 2 * 4 * 3 * vh * sizeof(float4))) != cudaSuccess)
-    return cuda_check(ctx, e, "cudaMalloc(gauge r12)");
-  if (!gc.u8 && (e = cudaMalloc(&gc.u8, 2 * 4 * 2 * vh * sizeof(float4))) != cudaSuccess)
-    return cuda_check(ctx, e, "cudaMalloc(gauge r8)");
-  if (!gc.u16 && (e = cudaMalloc(&gc.u16, 2 * 4 * 24 * vh)) != cudaSuccess)
-    return cuda_check(ctx, e, "cudaMalloc(gauge l16)");
-  if (!gc.u32lo && (e = cudaMalloc(&gc.u32lo, 2 * 4 * 18 * vh * sizeof(float))) != cudaSuccess)
-    return cuda_check(ctx, e, "cudaMalloc(gauge fp32 rounding errors)");
+  if (!gc.block) {
+    // one allocation for all copies; the digits of the FP64 Dslash last, left out where they would take more
+    // than a quarter of what is free (the Dslash works without them, slower)
+    const size_t bytes[] = {2 * 4 * 9 * vh * sizeof(double2), 2 * 4 * 18 * vh * sizeof(float),
+                            2 * 4 * 18 * vh * sizeof(float),  2 * 4 * 3 * vh * sizeof(float4),
+                            2 * 4 * 2 * vh * sizeof(float4),  2 * 4 * 24 * vh};
+    size_t off[7] = {0};
+    for (int j = 0; j < 6; ++j) off[j + 1] = (off[j] + bytes[j] + 255) / 256 * 256;
+    const size_t digits = 2 * 4 * fix_block_entries(g.vh) * sizeof(int4);
+    bool fix = true;
+    if (digits > (1u << 30)) {
+      size_t left = 0, total = 0;
+      if ((e = cudaMemGetInfo(&left, &total)) != cudaSuccess) return cuda_check(ctx, e, "cudaMemGetInfo");
+      fix = left > off[6] && digits <= (left - off[6]) / 4;
+    }
+    e = cudaMalloc(&gc.block, off[6] + (fix ? digits : 0));
+    if (e == cudaErrorMemoryAllocation && fix) {
+      cudaGetLastError();
+      fix = false;
+      e = cudaMalloc(&gc.block, off[6]);
+    }
+    if (e != cudaSuccess) {
+      gc.block = nullptr;
+      return cuda_check(ctx, e, "cudaMalloc(gauge field)");
+    }
+    char* at = static_cast<char*>(gc.block);
+    gc.u64 = reinterpret_cast<double2*>(at + off[0]);
+    gc.u32 = reinterpret_cast<float*>(at + off[1]);
+    gc.u32lo = reinterpret_cast<float*>(at + off[2]);
+    gc.u12 = reinterpret_cast<float4*>(at + off[3]);
+    gc.u8 = reinterpret_cast<float4*>(at + off[4]);
+    gc.u16 = at + off[5];
+    if (fix) gc.ufix = reinterpret_cast<int4*>(at + off[6]);
+  }
   e = launch_pack_gauge(g, reinterpret_cast<const double2*>(U_dev), gc, ctx->stream);
   ctx->launches += 1;
   if (e != cudaSuccess) return cuda_check(ctx, e, "pack_gauge");
@@ -243,7 +256,7 @@ int dslash_eo(lqcd_ctx* ctx, void* out_dev, const void* in_dev, int out_parity, 
 
 static const void* link_copy(const GaugeCopies& gc, int prec) {
   switch (prec) {
-    case LQCD_FP64: return gc.u64;
+    case LQCD_FP64: return gc.ufix;
     case LQCD_FP32_R12: return gc.u12;
     case LQCD_FP32_R8: return gc.u8;
     case LQCD_FP32_L16: return gc.u16;
@@ -282,6 +295,7 @@ int dslash_eo_batch(lqcd_ctx* const* ctxs, void* const* out_devs, const void* co
     const lqcd_ctx* c = ctxs[l];
     tab.lat[l].g = make_geom(c);
     tab.lat[l].links = link_copy(c->gauge, prec);
+    tab.lat[l].links64 = c->gauge.u64;
     tab.lat[l].in = in_devs[l];
     tab.lat[l].out = out_devs[l];
     tab.lat[l].out_parity = out_parities[l];
@@ -320,6 +334,7 @@ int dslash_eo_batch(lqcd_ctx* const* ctxs, void* const* out_devs, const void* co
       const lqcd_ctx* c = ctxs[l0 + j];
       a.lat[j].g = make_geom(c);
       a.lat[j].links = link_copy(c->gauge, prec);
+      a.lat[j].links64 = c->gauge.u64;
       a.lat[j].in = in_devs[l0 + j];
       a.lat[j].out = out_devs[l0 + j];
       a.lat[j].out_parity = out_parities[l0 + j];

@@ -13,14 +13,17 @@
 #include <string.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "internal.h"
 
 namespace lqcd {
 
 enum LinkFmt { kL64 = 0, kL32 = 1, kL12 = 2, kL8 = 3, kL16 = 4 };  // kL12 and up: signs applied after loading
+
+constexpr int kSMs = 152;         // GB300
+constexpr int kFixResident = 3;  // blocks per SM of the FP64 kernels (168 registers per thread)
 
 struct KArgs {
   void* out;
@@ -36,23 +39,15 @@ struct KArgs {
   double* partials;
   unsigned* ticket;
   const void* links;
+  const double2* links64;  // FP64 only: the copy behind the fixed-point one
   int order;  // block-to-site order (site_block)
-};
-
-template <int LF>
-struct LinkTraits {
-  typedef float T;
-};
-template <>
-struct LinkTraits<kL64> {
-  typedef double T;
 };
 
 // A link as loaded from memory (the compact forms stay compact while their loads are in flight)
 // and its decoding into a 3x3 matrix scaled by 1/2 * sign (signs are folded into L64 and L32).
 template <int LF>
 struct RawLink {
-  Mat3<typename LinkTraits<LF>::T> m;
+  Mat3<float> m;
 };
 template <>
 struct RawLink<kL12> {
@@ -71,9 +66,7 @@ struct RawLink<kL16> {
 template <int LF>
 __device__ __forceinline__ RawLink<LF> load_raw(const void* links, int p, int mu, int i, int vh, uint64_t pol) {
   RawLink<LF> r;
-  if constexpr (LF == kL64) {
-    r.m = load_link64(static_cast<const double2*>(links), p, mu, i, vh, pol);
-  } else if constexpr (LF == kL32) {
+  if constexpr (LF == kL32) {
     r.m = load_link32(static_cast<const float*>(links), p, mu, i, vh, pol);
   } else if constexpr (LF == kL12) {
     const float4* blk = static_cast<const float4*>(links) + (size_t)(p * 4 + mu) * 3 * vh;
@@ -93,8 +86,8 @@ __device__ __forceinline__ RawLink<LF> load_raw(const void* links, int p, int mu
 }
 
 template <int LF>
-__device__ __forceinline__ Mat3<typename LinkTraits<LF>::T> decode(const RawLink<LF>& r, int sign) {
-  if constexpr (LF == kL64 || LF == kL32) return r.m;
+__device__ __forceinline__ Mat3<float> decode(const RawLink<LF>& r, int sign) {
+  if constexpr (LF == kL32) return r.m;
   else if constexpr (LF == kL12) return decode_link12(r.a, r.b, r.c, 0.5f * (float)sign);
   else if constexpr (LF == kL8) return decode_link8(r.a, r.b, 0.5f * (float)sign);
   else return decode_link16(r.a, r.b, 0.5f * (float)sign);
@@ -107,6 +100,26 @@ __device__ __forceinline__ bool lane_writes(int sub, int c) {
   if (TPS == 1) return true;
   if (TPS == 2) return sub == 0 ? (c != 1) : (c == 1);
   return c == sub;
+}
+
+// The sum of the threads' dsite over the grid (every thread of the block calls).
+template <typename T>
+__device__ __forceinline__ void dslash_reduce(const KArgs& k, T dsite) {
+  if (!k.ticket) {  // the next kernel sums the per-block partials itself (FP32: as (hi, lo) pairs)
+    if constexpr (sizeof(T) == 4) {
+      const float2 bs = block_sum_f_df(dsite);
+      if (threadIdx.x == 0) reinterpret_cast<float2*>(k.partials)[blockIdx.x] = bs;
+    } else {
+      const double bs = block_sum_mixed(dsite);
+      if (threadIdx.x == 0) k.partials[blockIdx.x] = bs;
+    }
+    return;
+  }
+  double bs = block_sum_mixed(dsite);
+  if (publish_partial(k.partials, k.ticket, bs)) {
+    double tot = gather_partials(k.partials, k.ticket);
+    if (threadIdx.x == 0 && k.dot_out) *k.dot_out = tot;
+  }
 }
 
 // Output stage shared by the Dslash kernels: d = (D in)(x) of site i, written as the plain
@@ -151,23 +164,7 @@ __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d
       }
     }
   }
-  if constexpr (EPI != (int)Epi::Plain) {
-    if (!k.ticket) {  // the next kernel sums the per-block partials itself (FP32: as (hi, lo) pairs)
-      if constexpr (sizeof(T) == 4) {
-        const float2 bs = block_sum_f_df(dsite);
-        if (threadIdx.x == 0) reinterpret_cast<float2*>(k.partials)[blockIdx.x] = bs;
-      } else {
-        const double bs = block_sum_mixed(dsite);
-        if (threadIdx.x == 0) k.partials[blockIdx.x] = bs;
-      }
-      return;
-    }
-    double bs = block_sum_mixed(dsite);
-    if (publish_partial(k.partials, k.ticket, bs)) {
-      double tot = gather_partials(k.partials, k.ticket);
-      if (threadIdx.x == 0 && k.dot_out) *k.dot_out = tot;
-    }
-  }
+  if constexpr (EPI != (int)Epi::Plain) dslash_reduce<T>(k, dsite);
 }
 
 // The hops of lane `sub` of output site i (TPS lanes per site): h = sub, sub + TPS, ...; h even
@@ -178,8 +175,8 @@ __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d
 // returns the lane's share of (D in)(x).  Shared by the single-lattice and the batched kernels.
 template <int LF, int TPS>
 struct SiteHops {
-  typedef typename LinkTraits<LF>::T T;
-  typedef typename std::conditional<LF == kL64, double2, float2>::type V2;
+  typedef float T;
+  typedef float2 V2;
   static constexpr int NH = 8 / TPS;
   int nb[NH], sg[NH];
   RawLink<LF> Wn;
@@ -229,12 +226,6 @@ struct SiteHops {
   }
 };
 
-// FP32 links stay in L2 between launches; the FP64 copy (reliable updates) must not displace them
-template <int LF>
-__device__ __forceinline__ uint64_t link_policy() {
-  return (LF == kL64) ? policy_evict_first() : policy_evict_last();
-}
-
 // The chunk of output sites block blockIdx.x works on.  order 0: chunk b = block b (lexicographic
 // within the parity, the order of the stored vectors); order 1: the two halves of the site range
 // interleaved, even blocks taking the first half and odd blocks the second, so that blocks that run
@@ -249,8 +240,8 @@ __device__ __forceinline__ int site_block(int order) {
 
 template <int LF, int TPS, int EPI>
 __global__ void __launch_bounds__(128, 7) dslash_kernel(Geom g, KArgs k) {
-  typedef typename LinkTraits<LF>::T T;
-  typedef typename std::conditional<LF == kL64, double2, float2>::type V2;
+  typedef float T;
+  typedef float2 V2;
   const int vh = g.vh;
   const int gt = site_block(k.order) * blockDim.x + threadIdx.x;
   const int i = gt / TPS;
@@ -258,7 +249,7 @@ __global__ void __launch_bounds__(128, 7) dslash_kernel(Geom g, KArgs k) {
   const bool valid = i < vh;
   const int p = k.out_parity;
   const V2* in = static_cast<const V2*>(k.in);
-  const uint64_t pol = link_policy<LF>();
+  const uint64_t pol = policy_evict_last();
   SiteHops<LF, TPS> hops;
   // links are never written by the kernels of a solve: the first one is fetched before the wait
   if (valid) hops.start(g, k.links, p, i, sub, pol);
@@ -285,6 +276,57 @@ __global__ void __launch_bounds__(128, 7) dslash_kernel(Geom g, KArgs k) {
   dslash_epilogue<T, V2, TPS, EPI>(k, d, i, sub, valid, vh);
 }
 
+// FP64: the products in block fixed point (fix64.cuh), one direction per thread.  Blocks take groups of
+// kFixSites sites in turn; the next group's forward links are in flight while a group is finished.
+template <int EPI>
+__global__ void __launch_bounds__(kFixThreads, kFixResident) dslash64_kernel(Geom g, KArgs k) {
+  __shared__ FixShared sh;
+  const int vh = g.vh;
+  const int mu = threadIdx.x / kFixSites, ls = threadIdx.x % kFixSites;
+  const int p = k.out_parity;
+  const double2* in = static_cast<const double2*>(k.in);
+  const int4* U = static_cast<const int4*>(k.links);
+  const uint64_t pol = policy_evict_first();  // 8 % faster than evict_last, or than keeping part of them
+  const int step = gridDim.x * kFixSites;
+  int i = blockIdx.x * kFixSites + ls;
+  FixGroup grp;
+  if (i < vh) grp.start(g, U, p, i, mu, pol);
+  pdl_wait();
+  pdl_trigger();
+  if (k.done && *k.done) return;  // uniform: the flag only changes between kernels
+  const double a = k.a_dev ? *k.a_dev : k.a;
+  double2* out = static_cast<double2*>(k.out);
+  double dsite = 0.0;
+  for (int i0 = blockIdx.x * kFixSites; i0 < vh; i0 += step, i += step) {
+    const bool valid = i < vh, mine = valid && mu < 3;
+    const size_t o = (size_t)mu * vh + i;
+    double2 ps, bv;  // the epilogue's own-site loads, in flight beside the neighbours'
+    if constexpr (EPI != (int)Epi::Plain)
+      if (mine) ps = static_cast<const double2*>(k.aux)[o];
+    if constexpr (EPI == (int)Epi::Resid)
+      if (mine) bv = static_cast<const double2*>(k.bvec)[o];
+    grp.hops(sh, g, U, in, p, mu, ls, valid, pol);
+    if (i + step < vh) grp.start(g, U, p, i + step, mu, pol);
+    __syncthreads();
+    if (mine) {
+      const Cplx<double> d = FixGroup::colour(sh, g, U, k.links64, in, p, i, mu, ls);
+      double2 w = make_double2(d.re, d.im);
+      if constexpr (EPI != (int)Epi::Plain) {
+        w = make_double2(a * ps.x - d.re, a * ps.y - d.im);
+        if constexpr (EPI == (int)Epi::AApply) {
+          dsite += ps.x * w.x + ps.y * w.y;
+        } else {
+          w = make_double2(bv.x - w.x, bv.y - w.y);
+          dsite += w.x * w.x + w.y * w.y;
+        }
+      }
+      out[o] = w;
+    }
+    __syncthreads();  // sh is written again in the next turn
+  }
+  if constexpr (EPI != (int)Epi::Plain) dslash_reduce<double>(k, dsite);
+}
+
 // The half-lattice hop of NS systems that share one operator (the right-hand sides of a multi-RHS
 // shifted solve): every link is loaded and decoded once and applied to the NS input vectors, so the
 // link traffic per system drops by NS.  One thread per output site; per system the arithmetic (the
@@ -293,14 +335,14 @@ __global__ void __launch_bounds__(128, 7) dslash_kernel(Geom g, KArgs k) {
 template <int LF, int NS, int EPI>
 __global__ void __launch_bounds__(128, NS <= 2 ? 4 : 3) dslash_msys_kernel(Geom g,
                                                                           const __grid_constant__ PerSys<KArgs> pk) {
-  typedef typename LinkTraits<LF>::T T;
-  typedef typename std::conditional<LF == kL64, double2, float2>::type V2;
+  typedef float T;
+  typedef float2 V2;
   const int vh = g.vh;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = i < vh;
   const int p = pk.s[0].out_parity;
   const void* links = pk.s[0].links;
-  const uint64_t pol = link_policy<LF>();
+  const uint64_t pol = policy_evict_last();
   SiteHops<LF, 1> hops;
   if (valid) hops.start(g, links, p, i, 0, pol);
   pdl_wait();
@@ -356,16 +398,17 @@ __global__ void __launch_bounds__(128, NS <= 2 ? 4 : 3) dslash_msys_kernel(Geom 
 constexpr int kBatchChunk = 128;
 static_assert(sizeof(BatchArgs) <= 4000, "the batch descriptors travel as the kernel's parameter block");
 static_assert(kBatchPerLaunch <= kBatchChunk, "one thread per descriptor");
+static_assert(kFixThreads == kBatchChunk, "the FP64 groups use the whole block");
 
 // The persistent loop shared by both batched kernels: blocks take 128-site chunks of any lattice
 // from the work counter until none are left (lat and chunk_end already in shared memory).
 template <int LF>
 __device__ __forceinline__ void batch_loop(const BatchLattice* lat, const int* chunk_end, int n, unsigned* head,
                                            int* item_s) {
-  typedef typename LinkTraits<LF>::T T;
-  typedef typename std::conditional<LF == kL64, double2, float2>::type V2;
+  typedef float T;
+  typedef float2 V2;
   const int n_items = chunk_end[n];
-  const uint64_t pol = link_policy<LF>();
+  const uint64_t pol = policy_evict_last();
   for (;;) {
     if (threadIdx.x == 0) *item_s = (int)atomicAdd(head, 1u);
     __syncthreads();
@@ -384,18 +427,32 @@ __device__ __forceinline__ void batch_loop(const BatchLattice* lat, const int* c
     }
     if (l >= n) continue;
     const BatchLattice& L = lat[l];
-    const int i = (it - chunk_end[l]) * kBatchChunk + threadIdx.x;
-    if (i >= 0 && i < L.g.vh) {
-      SiteHops<LF, 1> hops;
-      hops.start(L.g, L.links, L.out_parity, i, 0, pol);
-      const Vec3<T> d = hops.apply(L.links, static_cast<const V2*>(L.in), L.out_parity, i, 0, L.g.vh, pol);
-      V2* out = static_cast<V2*>(L.out);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        V2 w;
-        w.x = d.c[c].re;
-        w.y = d.c[c].im;
-        out[(size_t)c * L.g.vh + i] = w;
+    const int i0 = (it - chunk_end[l]) * kBatchChunk;
+    if constexpr (LF == kL64) {
+      __shared__ FixShared sh;
+      const int mu = threadIdx.x / kFixSites, ls = threadIdx.x % kFixSites, vh = L.g.vh, p = L.out_parity;
+      const int4* U = static_cast<const int4*>(L.links);
+      const double2* in = static_cast<const double2*>(L.in);
+      for (int j0 = i0; j0 < min(i0 + kBatchChunk, vh); j0 += kFixSites) {
+        const int i = j0 + ls;
+        const bool valid = i < vh;
+        FixGroup grp;
+        if (valid) grp.start(L.g, U, p, i, mu, pol);
+        grp.hops(sh, L.g, U, in, p, mu, ls, valid, pol);
+        __syncthreads();
+        if (valid && mu < 3) {
+          const Cplx<double> d = FixGroup::colour(sh, L.g, U, L.links64, in, p, i, mu, ls);
+          static_cast<double2*>(L.out)[(size_t)mu * vh + i] = make_double2(d.re, d.im);
+        }
+        __syncthreads();
+      }
+    } else {
+      const int i = i0 + threadIdx.x;
+      if (i >= 0 && i < L.g.vh) {
+        SiteHops<LF, 1> hops;
+        hops.start(L.g, L.links, L.out_parity, i, 0, pol);
+        const Vec3<T> d = hops.apply(L.links, static_cast<const V2*>(L.in), L.out_parity, i, 0, L.g.vh, pol);
+        store_vec(static_cast<V2*>(L.out), i, L.g.vh, d);
       }
     }
   }
@@ -403,7 +460,8 @@ __device__ __forceinline__ void batch_loop(const BatchLattice* lat, const int* c
 
 // descriptors in the parameter block (up to kBatchPerLaunch lattices), copied to shared memory
 template <int LF>
-__global__ void __launch_bounds__(kBatchChunk, 7) dslash_batch_kernel(BatchArgs a, unsigned* head) {
+__global__ void __launch_bounds__(kBatchChunk, LF == kL64 ? kFixResident : 7)
+    dslash_batch_kernel(BatchArgs a, unsigned* head) {
   __shared__ BatchLattice lat[kBatchPerLaunch];
   __shared__ int chunk_end[kBatchPerLaunch + 1];
   __shared__ int item_s;
@@ -421,8 +479,8 @@ __global__ void __launch_bounds__(kBatchChunk, 7) dslash_batch_kernel(BatchArgs 
 
 // descriptors in a device table (up to kMaxBatch lattices), copied to shared memory
 template <int LF>
-__global__ void __launch_bounds__(kBatchChunk, 7) dslash_batch_table_kernel(const BatchTable* __restrict__ tab,
-                                                                             unsigned* head) {
+__global__ void __launch_bounds__(kBatchChunk, LF == kL64 ? kFixResident : 7)
+    dslash_batch_table_kernel(const BatchTable* __restrict__ tab, unsigned* head) {
   __shared__ BatchLattice lat[kMaxBatch];
   __shared__ int chunk_end[kMaxBatch + 1];
   __shared__ int item_s;
@@ -441,7 +499,8 @@ cudaError_t launch_dslash_batch(const BatchArgs& a, int prec, unsigned* head, in
   if (items <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(head, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::min(items, 7 * n_sm);  // one resident wave of persistent blocks
+  // one resident wave of persistent blocks
+  const unsigned grid = (unsigned)std::min(items, (prec == LQCD_FP64 ? kFixResident : 7) * n_sm);
   switch (prec) {
     case LQCD_FP64: dslash_batch_kernel<kL64><<<grid, kBatchChunk, 0, st>>>(a, head); break;
     case LQCD_FP32_R12: dslash_batch_kernel<kL12><<<grid, kBatchChunk, 0, st>>>(a, head); break;
@@ -457,7 +516,8 @@ cudaError_t launch_dslash_batch_table(const BatchTable* tab, int n_items, int pr
   if (n_items <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(head, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::min(n_items, 7 * n_sm);  // one resident wave of persistent blocks
+  // one resident wave of persistent blocks
+  const unsigned grid = (unsigned)std::min(n_items, (prec == LQCD_FP64 ? kFixResident : 7) * n_sm);
   switch (prec) {
     case LQCD_FP64: dslash_batch_table_kernel<kL64><<<grid, kBatchChunk, 0, st>>>(tab, head); break;
     case LQCD_FP32_R12: dslash_batch_table_kernel<kL12><<<grid, kBatchChunk, 0, st>>>(tab, head); break;
@@ -481,24 +541,33 @@ static cudaError_t launch_tps(const Geom& g, const KArgs& k, Epi epi, cudaStream
 
 template <int LF>
 static cudaError_t launch_lf(const Geom& g, const KArgs& k, Epi epi, int tps, int bs, cudaStream_t st, bool pdl) {
-  if constexpr (LF == kL64) {
-    return launch_tps<LF, 1>(g, k, epi, st, 128, pdl);  // FP64 is arithmetic-bound: one thread per site
-  } else {
-    switch (tps) {
-      case 1: return launch_tps<LF, 1>(g, k, epi, st, bs, pdl);
-      case 2: return launch_tps<LF, 2>(g, k, epi, st, bs, pdl);
-      case 4: return launch_tps<LF, 4>(g, k, epi, st, bs, pdl);
-      default: return launch_tps<LF, 8>(g, k, epi, st, bs, pdl);
-    }
+  switch (tps) {
+    case 1: return launch_tps<LF, 1>(g, k, epi, st, bs, pdl);
+    case 2: return launch_tps<LF, 2>(g, k, epi, st, bs, pdl);
+    case 4: return launch_tps<LF, 4>(g, k, epi, st, bs, pdl);
+    default: return launch_tps<LF, 8>(g, k, epi, st, bs, pdl);
+  }
+}
+
+// FP64 blocks: one per group of sites, at most one resident wave (the blocks then take several groups each)
+static int fp64_blocks(const Geom& g) { return std::min((g.vh + kFixSites - 1) / kFixSites, kFixResident * kSMs); }
+
+static cudaError_t launch_fp64(const Geom& g, const KArgs& k, Epi epi, cudaStream_t st, bool pdl) {
+  const dim3 nb((unsigned)fp64_blocks(g)), bs(kFixThreads);
+  switch (epi) {
+    case Epi::Plain: return launch_k(pdl, dslash64_kernel<0>, nb, bs, st, g, k);
+    case Epi::AApply: return launch_k(pdl, dslash64_kernel<1>, nb, bs, st, g, k);
+    default: return launch_k(pdl, dslash64_kernel<2>, nb, bs, st, g, k);
   }
 }
 
 static int default_tps(int) { return 1; }  // fastest on GB300 at 16^3x8 and 32^3x8 (sweep over 1, 2, 4, 8)
 
-// blocks of one Dslash launch (= partials it writes): the FP64 kernel always runs 1 thread per site
+// blocks of one Dslash launch (= partials it writes)
 int dslash_grid_blocks(const Geom& g, int prec, int tps, int bs) {
-  if (tps <= 0 || prec == LQCD_FP64) tps = default_tps(prec);
-  if (bs <= 0 || prec == LQCD_FP64) bs = 128;
+  if (prec == LQCD_FP64) return fp64_blocks(g);
+  if (tps <= 0) tps = default_tps(prec);
+  if (bs <= 0) bs = 128;
   long long threads = (long long)g.vh * tps;
   return (int)((threads + bs - 1) / bs);
 }
@@ -524,7 +593,10 @@ cudaError_t launch_dslash(const Geom& g, const GaugeCopies& gc, const DslashArgs
   k.order = (a.prec == LQCD_FP64) ? 0 : a.order;
   if (nlaunch) *nlaunch += 1;
   switch (a.prec) {
-    case LQCD_FP64: k.links = gc.u64; return launch_lf<kL64>(g, k, a.epi, tps, bs, st, a.pdl);
+    case LQCD_FP64:
+      k.links = gc.ufix;
+      k.links64 = gc.u64;
+      return launch_fp64(g, k, a.epi, st, a.pdl);
     case LQCD_FP32_R12: k.links = gc.u12; return launch_lf<kL12>(g, k, a.epi, tps, bs, st, a.pdl);
     case LQCD_FP32_R8: k.links = gc.u8; return launch_lf<kL8>(g, k, a.epi, tps, bs, st, a.pdl);
     case LQCD_FP32_L16: k.links = gc.u16; return launch_lf<kL16>(g, k, a.epi, tps, bs, st, a.pdl);

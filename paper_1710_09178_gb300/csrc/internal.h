@@ -84,7 +84,9 @@ struct SolverDev {
 };
 
 struct GaugeCopies {
+  void* block = nullptr;   // the allocation that holds the copies
   double2* u64 = nullptr;  // [2][4][9][Vh] double2, 1/2 eta*bc folded in
+  int4* ufix = nullptr;    // the digits of u64 (fix64.cuh), null where there is no room for them
   float* u32 = nullptr;    // [2][4][18][Vh] floats (float4 x4 + float2), 1/2 eta*bc folded in
   float4* u12 = nullptr;   // [2][4][3][Vh] float4, rows 0-1, no sign
   float4* u8 = nullptr;    // [2][4][2][Vh] float4, 8-real form, no sign
@@ -185,6 +187,7 @@ constexpr int kBatchPerLaunch = 32;
 struct BatchLattice {
   Geom g;
   const void* links;  // the link copy of the batch's precision
+  const double2* links64;  // FP64: the copy behind the fixed-point one
   const void* in;
   void* out;
   int out_parity;

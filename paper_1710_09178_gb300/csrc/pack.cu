@@ -1,6 +1,7 @@
 // pack.cu - conversion between the canonical boundary layouts and the internal
 // structure-of-arrays layouts, and the written-out neighbour tables.
 #include "common.cuh"
+#include "fix64.cuh"
 #include "internal.h"
 
 namespace lqcd {
@@ -24,9 +25,10 @@ __device__ __forceinline__ int pack_codes(double re, double im) {
   return (qr & 0xffff) | (qi << 16);
 }
 
-// One thread per (site, mu): canonical complex128 [V][4][3][3] -> five internal copies.
+// One thread per (site, mu): canonical complex128 [V][4][3][3] -> the internal copies.
 __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2* __restrict__ u64,
-                                  float* __restrict__ u32, float4* __restrict__ u12, float4* __restrict__ u8,
+                                  int4* __restrict__ ufix, float* __restrict__ u32, float4* __restrict__ u12,
+                                  float4* __restrict__ u8,
                                   char* __restrict__ u16, float* __restrict__ u32lo) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   long long V = 2LL * g.vh;
@@ -45,6 +47,24 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
     double2* b = u64 + (size_t)(p * 4 + mu) * 9 * vh + i;
 #pragma unroll
     for (int j = 0; j < 9; ++j) b[(size_t)j * vh] = make_double2(half_sign * e[j].x, half_sign * e[j].y);
+  }
+  if (ufix) {
+    int4* b = ufix + fix_entry(p, mu, i, vh);
+    double2 u[9];
+#pragma unroll
+    for (int j = 0; j < 9; ++j) u[j] = make_double2(half_sign * e[j].x, half_sign * e[j].y);
+    const bool fits = fix_link_fits(u);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      int4 w = make_int4(0, 0, 0, 0);
+      if (fits) {
+        const Fix2 re = fix_link_entry(u[j].x), im = fix_link_entry(u[j].y);
+        w = make_int4(re.h, re.l, im.h, im.l);
+      } else if (j == 0) {
+        w.x = kFixBadLink;
+      }
+      b[j * 32] = w;
+    }
   }
   if (u32) {
     float* blk = u32 + (size_t)(p * 4 + mu) * 18 * vh;
@@ -102,7 +122,7 @@ cudaError_t launch_pack_gauge(const Geom& g, const double2* U, GaugeCopies& gc, 
   long long n = 8LL * g.vh;  // 4 V threads
   int bs = 256;
   long long nb = (n + bs - 1) / bs;
-  pack_gauge_kernel<<<(unsigned)nb, bs, 0, st>>>(g, U, gc.u64, gc.u32, gc.u12, gc.u8, gc.u16, gc.u32lo);
+  pack_gauge_kernel<<<(unsigned)nb, bs, 0, st>>>(g, U, gc.u64, gc.ufix, gc.u32, gc.u12, gc.u8, gc.u16, gc.u32lo);
   return cudaGetLastError();
 }
 
