@@ -53,11 +53,12 @@ DSLASH_BYTES_PER_SITE = {"fp32": 8 * 72 + 24 + 24, "fp32_r12": 8 * 48 + 24 + 24,
                          "fp32_l16": 8 * 24 + 24 + 24, "fp64": 8 * 144 + 48 + 48}
 DSLASH_FLOPS_PER_SITE = 570
 # The double-FP32 half Dslash (the checks and the first phase of the mixed solve): per output site 8 hops x
-# 9 link entries x 4 real products, each one compensated multiply-add of 12 FP32 operations (product,
-# its exact error and the two cross terms: 4; TwoSum into the running sum: 6; the compensation: 2), and
-# 6 final renormalisations of 2; bytes, counted as for the FP32 Dslash (each crossing HBM once): 8 link
-# pairs (hi, lo: 2 x 72), the input pair (2 x 24, re-read from L2 by the neighbours) and the output pair
-DF_OPS_PER_SITE = 8 * 9 * 4 * 12 + 6 * 2
+# 9 link entries x 4 real products, each one compensated multiply-add of 10 FP32 operations (the product;
+# TwoSum into the running sum with the exact product's remainder: 6; the cross terms: 2; the compensation:
+# 1), 3 x 6 additions of the directions' sums of 8, and 6 final renormalisations of 2;
+# bytes, counted as for the FP32 Dslash (each crossing HBM once): 8 link pairs (hi, lo: 2 x 72), the input pair
+# (2 x 24, re-read from L2 by the neighbours) and the output pair
+DF_OPS_PER_SITE = 8 * 9 * 4 * 10 + 3 * 6 * 8 + 6 * 2
 DF_BYTES_PER_SITE = 8 * 144 + 48 + 48
 
 

@@ -582,18 +582,21 @@ __device__ __forceinline__ Mat3<float> decode_link16(int4 a, int2 b, float scale
 // Double-FP32 ("df") arithmetic: an FP64-class number as an FP32 pair (hi, lo), operated on
 // with FP32 instructions only (exact FMA products, Knuth's TwoSum).
 // ---------------------------------------------------------------------------
-// s + c += (ah + al)(bh + bl), dropping al bl.  The _rn intrinsics are never contracted into
-// fused multiply-adds, which TwoSum's exactness requires.
+// s + c += (ah + al)(bh + bl), dropping al bl.  p = fl(ah bh) enters s by Knuth's TwoSum, whose error is
+// (s - (t - z)) + (p - z); the exact product's remainder past z, ah bh - z = (p - z) + (ah bh - p), takes one fma
+// instead of a subtraction and a product error: it is at most an ulp of t, so its rounding is 2^-48 of the
+// sum.  10 operations.  The _rn intrinsics are never contracted into fused multiply-adds, which TwoSum's
+// exactness requires.
 __device__ __forceinline__ void df_mac(float& s, float& c, float ah, float al, float bh, float bl) {
   const float p = __fmul_rn(ah, bh);
-  float e = __fmaf_rn(ah, bh, -p);
-  e = __fmaf_rn(ah, bl, e);
-  e = __fmaf_rn(al, bh, e);
   const float t = __fadd_rn(s, p);
   const float z = __fsub_rn(t, s);
-  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
+  const float d = __fsub_rn(s, __fsub_rn(t, z));
+  float e = __fmaf_rn(ah, bh, -z);
+  e = __fmaf_rn(ah, bl, e);
+  e = __fmaf_rn(al, bh, e);
   s = t;
-  c = __fadd_rn(c, __fadd_rn(err, e));
+  c = __fadd_rn(c, __fadd_rn(d, e));
 }
 
 // s + c += (bh + bl)

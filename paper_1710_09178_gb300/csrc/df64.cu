@@ -7,11 +7,10 @@
 // FP64 Dslash is arithmetic-bound at ~75 us on 32^3 x 8.  Here the same residual is computed
 // with FP32 instructions only:
 //   - every FP64 number u is held as a pair (hi, lo) = (fl32(u), fl32(u - hi)) (about 48 bits);
-//   - a product (ah + al)(bh + bl) is p + e with p = fl32(ah bh) and its exact rounding error
-//     fma(ah, bh, -p) plus the cross terms ah bl + al bh (al bl, ~2^-48 relative, is dropped);
-//   - p enters the running sum s through Knuth's TwoSum (s + p = t + err exactly) and err + e
-//     go to a compensation c, so s + c carries the sum to ~2^-48 relative to the sum of the
-//     magnitudes of its terms.
+//   - of a product (ah + al)(bh + bl), p = fl32(ah bh) enters the running sum s through Knuth's TwoSum; what
+//     s does not take (TwoSum's error, the product's rounding and the cross terms ah bl + al bh; al bl,
+//     ~2^-48 relative, is dropped) goes to a compensation c, so s + c carries the sum to ~2^-48
+//     relative to the sum of the magnitudes of its terms (df_mac: 10 operations).
 // The links are the FP32 copy (hi, 1/2 eta bc folded in) plus a copy of the FP32 rounding
 // errors (lo); vectors are split from FP64 once per residual.  The result is rounded to FP32
 // (the reliable update and the refinement both continue in FP32) and |r|^2 is summed in FP64.
@@ -26,6 +25,8 @@
 #include "solver_dev.cuh"
 
 namespace lqcd {
+
+constexpr int kDfThreads = 128;  // of the Dslash; 4 blocks per SM (128 registers)
 
 // Sum over the block of per-thread double-FP32 values (s, c): TwoSum shuffles within each warp,
 // then the warps' FP64 values in a fixed order.  Result valid in thread 0 (which publishes it).
@@ -90,128 +91,163 @@ __device__ __forceinline__ void df_hop(float (&sr)[3], float (&cr)[3], float (&s
   }
 }
 
-// hop h of output site s (index i): the neighbour's index and the link's parity and index
-struct DfHopSite {
-  int j, lp, li, mu;
-  bool fwd;
-};
-__device__ __forceinline__ DfHopSite df_hop_site(const Geom& g, const Site& s, int p, int i, int h) {
-  DfHopSite o;
-  o.mu = h >> 1;
-  o.fwd = (h & 1) == 0;
-  o.j = neighbour_half(g, o.fwd ? neighbour_fwd(g, s, o.mu) : neighbour_bwd(g, s, o.mu));
-  o.lp = o.fwd ? p : 1 - p;
-  o.li = o.fwd ? i : o.j;
-  return o;
-}
-
 __device__ __forceinline__ float2 df_a(const DfArgs& k) {
   return k.a_split ? make_float2(k.a_hi, k.a_lo) : (k.a_devdf ? *k.a_devdf : split64(k.a_dev ? *k.a_dev : k.a));
 }
 
-// EPI 0 output of site i: D in as (hi, lo)
-__device__ __forceinline__ void df_store_plain(const DfArgs& k, int i, int vh, const float (&sr)[3],
-                                               const float (&cr)[3], const float (&si)[3], const float (&ci)[3]) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const float2 re = df_norm(sr[a], cr[a]), im = df_norm(si[a], ci[a]);
-    k.out_hi[(size_t)a * vh + i] = make_float2(re.x, im.x);
-    k.out_lo[(size_t)a * vh + i] = make_float2(re.y, im.y);
+// What the epilogues read at the output site beside the hops' sum, for one colour.
+struct DfOwn {
+  float2 xh, xl, bh, bl;
+};
+template <int EPI>
+__device__ __forceinline__ DfOwn df_own(const DfArgs& k, size_t o) {
+  DfOwn w;
+  if constexpr (EPI != 0) {
+    w.xh = k.x_hi[o];
+    w.xl = k.x_lo[o];
   }
+  if constexpr (EPI == 2) {
+    w.bh = k.b_hi[o];
+    w.bl = k.b_lo[o];
+  }
+  return w;
 }
 
-// EPI 2 at site i: r = fl32(b - a x + D in), stored when r_out is set; returns the site's |r|^2 (FP32)
-__device__ __forceinline__ float df_resid_site(const DfArgs& k, int i, int vh, const float (&sr)[3],
-                                               const float (&cr)[3], const float (&si)[3], const float (&ci)[3]) {
-  const float2 asp = df_a(k);
-  const float ah = asp.x, al = asp.y;
-  float dsite = 0.f;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const size_t o = (size_t)a * vh + i;
-    const float2 bh = k.b_hi[o], bl = k.b_lo[o], xh = k.x_hi[o], xl = k.x_lo[o];
-    float rs = bh.x, rc = bl.x, is = bh.y, ic = bl.y;
-    df_mac(rs, rc, -ah, -al, xh.x, xl.x);
-    df_mac(is, ic, -ah, -al, xh.y, xl.y);
-    df_add(rs, rc, sr[a], cr[a]);
-    df_add(is, ic, si[a], ci[a]);
+// One colour of the output at offset o, d = (sr + cr, si + ci) its D in:  EPI 0: out = d;  EPI 1: out = a x - d,
+// (ds, dc) += Re<x, out>;  EPI 2: r = fl32(b - (a x - d)) (stored unless r_out is null), ds += |r|^2.
+template <int EPI>
+__device__ __forceinline__ void df_finish(const DfArgs& k, size_t o, float2 asp, const DfOwn& w, float sr, float cr,
+                                          float si, float ci, float& ds, float& dc) {
+  if constexpr (EPI == 0) {
+    const float2 re = df_norm(sr, cr), im = df_norm(si, ci);
+    k.out_hi[o] = make_float2(re.x, im.x);
+    k.out_lo[o] = make_float2(re.y, im.y);
+  } else if constexpr (EPI == 1) {
+    float rs = 0.f, rc = 0.f, is = 0.f, ic = 0.f;
+    df_mac(rs, rc, asp.x, asp.y, w.xh.x, w.xl.x);
+    df_mac(is, ic, asp.x, asp.y, w.xh.y, w.xl.y);
+    df_add(rs, rc, -sr, -cr);
+    df_add(is, ic, -si, -ci);
+    const float2 re = df_norm(rs, rc), im = df_norm(is, ic);
+    k.out_hi[o] = make_float2(re.x, im.x);
+    k.out_lo[o] = make_float2(re.y, im.y);
+    df_mac(ds, dc, w.xh.x, w.xl.x, re.x, re.y);
+    df_mac(ds, dc, w.xh.y, w.xl.y, im.x, im.y);
+  } else {
+    float rs = w.bh.x, rc = w.bl.x, is = w.bh.y, ic = w.bl.y;
+    df_mac(rs, rc, -asp.x, -asp.y, w.xh.x, w.xl.x);
+    df_mac(is, ic, -asp.x, -asp.y, w.xh.y, w.xl.y);
+    df_add(rs, rc, sr, cr);
+    df_add(is, ic, si, ci);
     const float rr = __fadd_rn(rs, rc), ri = __fadd_rn(is, ic);
     if (k.r_out) k.r_out[o] = make_float2(rr, ri);
-    dsite += rr * rr + ri * ri;
+    ds += rr * rr + ri * ri;
   }
-  return dsite;
 }
 
-// EPI 0: out = D in (hi, lo);  EPI 1: out = a x - D in and Re<x, out> (the A-apply; inside the
-// solve, without a ticket, the sum stays as per-block (hi, lo) partials for the r update);
-// EPI 2: r_out = fl32(b - (a x - D in)) (unless r_out is null) and |r_out|^2 (FP64 sum).
+// the end of a site's sum: 0 plain, 1 the A-apply (inside the solve, without a ticket, the sum stays as
+// per-block (hi, lo) partials for the r update), 2 the residual
 template <int EPI>
-__global__ void __launch_bounds__(128, 4) df_dslash_kernel(Geom g, const __grid_constant__ PerSys<DfArgs> pk) {
-  const DfArgs& k = pk.s[blockIdx.y];  // system blockIdx.y
+__device__ __forceinline__ void df_reduce(const DfArgs& k, float ds, float dc) {
+  if constexpr (EPI == 0) return;
+  double bs;
+  if constexpr (EPI == 1) {
+    if (!k.ticket) {
+      const float2 b2 = block_sum_df_df(ds, dc);
+      if (threadIdx.x == 0) reinterpret_cast<float2*>(k.partials)[blockIdx.x] = b2;
+      return;
+    }
+    bs = block_sum_df(ds, dc);
+  } else {
+    bs = block_sum_mixed(ds);
+  }
+  if (publish_partial(k.partials, k.ticket, bs)) {
+    const double tot = gather_partials(k.partials, k.ticket);
+    if (threadIdx.x == 0 && k.dot_out) *k.dot_out = tot;
+  }
+}
+
+// The half Dslash of system blockIdx.y with its epilogue.  Every direction's pair of hops (forward, then
+// backward) is one double-FP32 sum, and the four are added in order, whatever TPS, so the bits do not
+// depend on how the directions are spread over threads.
+// The block holds NS = blockDim.x / TPS sites; thread t takes directions t / NS ND .. of site t % NS, ND = 4 / TPS.
+// The four sums meet in shared memory (which with TPS = 1 also keeps them out of the registers that the
+// next links are loaded into), and thread sub finishes colours sub, sub + TPS, ..
+template <int EPI, int TPS>
+__global__ void __launch_bounds__(kDfThreads, 4) df_dslash_kernel(Geom g, const __grid_constant__ PerSys<DfArgs> pk) {
+  constexpr int NS = kDfThreads / TPS, ND = 4 / TPS;
+  __shared__ float4 part[4][3][NS];
+  const DfArgs& k = pk.s[blockIdx.y];
   const int vh = g.vh;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int sub = threadIdx.x / NS, ls = threadIdx.x % NS;
+  const int i = blockIdx.x * NS + ls;
   const bool valid = i < vh;
   const int p = k.out_parity;
+  const uint64_t pol_hi = policy_evict_last();   // the solver's FP32 links: keep them in L2
+  const uint64_t pol_lo = policy_evict_first();  // rounding errors, read only by the checks
+  // With several threads per site the launch is short of work, and its latency counts: the first link (which no
+  // kernel of a solve writes) is fetched before the wait and the epilogue's vectors beside the hops'.
+  Mat3<float> Uh, Ul;
+  Site s;
+  if (valid) {
+    s = site_of(g, p, i);
+    if (TPS > 1) {
+      Uh = load_link32(k.links_hi, p, sub * ND, i, vh, pol_hi);
+      Ul = load_link32(k.links_lo, p, sub * ND, i, vh, pol_lo);
+    }
+  }
   pdl_wait();
   pdl_trigger();
   if ((k.done && *k.done) || (k.halt && *k.halt)) return;  // uniform
 
-  float sr[3] = {0.f, 0.f, 0.f}, cr[3] = {0.f, 0.f, 0.f}, si[3] = {0.f, 0.f, 0.f}, ci[3] = {0.f, 0.f, 0.f};
+  constexpr int NC = (3 + TPS - 1) / TPS;  // colours finished by thread sub: sub, sub + TPS, ..
+  DfOwn own[NC];
+  float2 asp = make_float2(0.f, 0.f);
+  auto load_own = [&]() {
+    if (EPI != 0) asp = df_a(k);
+#pragma unroll
+    for (int q = 0; q < NC; ++q)
+      if (valid && sub + q * TPS < 3) own[q] = df_own<EPI>(k, (size_t)(sub + q * TPS) * vh + i);
+  };
+  if (TPS > 1) load_own();
   if (valid) {
-    const Site s = site_of(g, p, i);
-    const uint64_t pol_hi = policy_evict_last();   // the solver's FP32 links: keep them in L2
-    const uint64_t pol_lo = policy_evict_first();  // rounding errors, read only by the checks
 #pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      const DfHopSite o = df_hop_site(g, s, p, i, h);
-      const Mat3<float> Uh = load_link32(k.links_hi, o.lp, o.mu, o.li, vh, pol_hi);
-      const Mat3<float> Ul = load_link32(k.links_lo, o.lp, o.mu, o.li, vh, pol_lo);
-      const Vec3<float> vh3 = ldg_vec(k.in_hi, o.j, vh), vl3 = ldg_vec(k.in_lo, o.j, vh);
-      df_hop(sr, cr, si, ci, Uh, Ul, vh3, vl3, o.fwd);
-    }
-  }
-  if constexpr (EPI == 0) {
-    if (valid) df_store_plain(k, i, vh, sr, cr, si, ci);
-  } else if constexpr (EPI == 1) {
-    // q = a x - D in (x = the own-site vector, p of the solve), Re<x, q> in double-FP32
-    float ds = 0.f, dc = 0.f;
-    if (valid) {
-      const float2 asp = df_a(k);
-      const float ah = asp.x, al = asp.y;
+    for (int d = 0; d < ND; ++d) {
+      float sr[3] = {0.f, 0.f, 0.f}, cr[3] = {0.f, 0.f, 0.f}, si[3] = {0.f, 0.f, 0.f}, ci[3] = {0.f, 0.f, 0.f};
+      const int mu = sub * ND + d;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const size_t o = (size_t)a * vh + i;
-        const float2 xh = k.x_hi[o], xl = k.x_lo[o];
-        float rs = 0.f, rc = 0.f, is = 0.f, ic = 0.f;
-        df_mac(rs, rc, ah, al, xh.x, xl.x);
-        df_mac(is, ic, ah, al, xh.y, xl.y);
-        df_add(rs, rc, -sr[a], -cr[a]);
-        df_add(is, ic, -si[a], -ci[a]);
-        const float2 re = df_norm(rs, rc), im = df_norm(is, ic);
-        k.out_hi[o] = make_float2(re.x, im.x);
-        k.out_lo[o] = make_float2(re.y, im.y);
-        df_mac(ds, dc, xh.x, xl.x, re.x, re.y);
-        df_mac(ds, dc, xh.y, xl.y, im.x, im.y);
+      for (int h = 0; h < 2; ++h) {
+        const bool fwd = h == 0;
+        const int j = neighbour_half(g, fwd ? neighbour_fwd(g, s, mu) : neighbour_bwd(g, s, mu));
+        const int lp = fwd ? p : 1 - p, li = fwd ? i : j;
+        if (TPS == 1 || d > 0 || h > 0) {
+          Uh = load_link32(k.links_hi, lp, mu, li, vh, pol_hi);
+          Ul = load_link32(k.links_lo, lp, mu, li, vh, pol_lo);
+        }
+        const Vec3<float> vh3 = ldg_vec(k.in_hi, j, vh), vl3 = ldg_vec(k.in_lo, j, vh);
+        df_hop(sr, cr, si, ci, Uh, Ul, vh3, vl3, fwd);
       }
-    }
-    if (!k.ticket) {  // inside the solve: the r update sums the (hi, lo) partials itself
-      const float2 bs = block_sum_df_df(ds, dc);
-      if (threadIdx.x == 0) reinterpret_cast<float2*>(k.partials)[blockIdx.x] = bs;
-      return;
-    }
-    const double bs = block_sum_df(ds, dc);
-    if (publish_partial(k.partials, k.ticket, bs)) {
-      const double tot = gather_partials(k.partials, k.ticket);
-      if (threadIdx.x == 0 && k.dot_out) *k.dot_out = tot;
-    }
-  } else {
-    const float dsite = valid ? df_resid_site(k, i, vh, sr, cr, si, ci) : 0.f;
-    const double bs = block_sum_mixed(dsite);
-    if (publish_partial(k.partials, k.ticket, bs)) {
-      const double tot = gather_partials(k.partials, k.ticket);
-      if (threadIdx.x == 0) *k.dot_out = tot;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) part[mu][c][ls] = make_float4(sr[c], cr[c], si[c], ci[c]);
     }
   }
+  if (TPS > 1) __syncthreads();
+  else load_own();
+  float ds = 0.f, dc = 0.f;
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    const int c = sub + q * TPS;
+    if (!valid || c >= 3) continue;
+    float4 t = part[0][c][ls];
+#pragma unroll
+    for (int mu = 1; mu < 4; ++mu) {
+      const float4 u = part[mu][c][ls];
+      df_add(t.x, t.y, u.x, u.y);
+      df_add(t.z, t.w, u.z, u.w);
+    }
+    df_finish<EPI>(k, (size_t)c * vh + i, asp, own[q], t.x, t.y, t.z, t.w, ds, dc);
+  }
+  df_reduce<EPI>(k, ds, dc);
 }
 
 cudaError_t launch_split_df(const Geom& g, const double2* x, float2* hi, float2* lo, const int* done, cudaStream_t st,
@@ -220,13 +256,36 @@ cudaError_t launch_split_df(const Geom& g, const double2* x, float2* hi, float2*
   return launch_k(pdl, split_df_kernel, dim3((n3 + 255) / 256), dim3(256), st, n3, x, hi, lo, done);
 }
 
-int df_dslash_grid_blocks(const Geom& g) { return (g.vh + 127) / 128; }
+// Threads per site: the most that keep the launch within two blocks per SM (304), so that a small lattice's chain
+// of eight hops is shortened while the SMs have room.  Half Dslash per graph launch, in us, with 1 / 2 / 4 threads
+// per site (12-operation df_mac): 8^4 6.3 / 3.2 / 2.4, 16^3x8 7.3 / 4.3 / 4.5, 24^3x6 9.8 / 9.5 / 11.2, 32^3x8
+// 24.2 / 25.7 / 30.6, 48^3x12 129 / 132 / 159 (A-applies at 24^3x6 23.5 / 25.9 / 32.4): more threads repeat the
+// site's index arithmetic.  One thread per colour instead gives 4.7, 5.7 and 10.8 us at the first three.
+// With everything here: 8^4 6.2 -> 2.35 us, 16^3x8 7.2 -> 4.05, 24^3x6 9.5 -> 9.8, 32^3x8 23.6 -> 24.5 (A-apply
+// 57.7 -> 56.7), error against quad precision 1.6e-14 -> 7.0e-15 (Gaussian vectors).
+static int df_tps(const Geom& g) {
+  constexpr int kBlocks = 304;
+  return g.vh <= kBlocks * kDfThreads / 4 ? 4 : (g.vh <= kBlocks * kDfThreads / 2 ? 2 : 1);
+}
+int df_dslash_grid_blocks(const Geom& g) {
+  const int ns = kDfThreads / df_tps(g);
+  return (g.vh + ns - 1) / ns;
+}
+
+template <int TPS>
+static cudaError_t launch_df_tps(const Geom& g, const PerSys<DfArgs>& a, int S, int epi, cudaStream_t st, bool pdl) {
+  const dim3 grid((unsigned)df_dslash_grid_blocks(g), (unsigned)S), block(kDfThreads);
+  if (epi == 2) return launch_k(pdl, df_dslash_kernel<2, TPS>, grid, block, st, g, a);
+  if (epi == 1) return launch_k(pdl, df_dslash_kernel<1, TPS>, grid, block, st, g, a);
+  return launch_k(pdl, df_dslash_kernel<0, TPS>, grid, block, st, g, a);
+}
 
 cudaError_t launch_df_dslash_multi(const Geom& g, const PerSys<DfArgs>& a, int S, int epi, cudaStream_t st, bool pdl) {
-  const dim3 grid((unsigned)df_dslash_grid_blocks(g), (unsigned)S);
-  if (epi == 2) return launch_k(pdl, df_dslash_kernel<2>, grid, dim3(128), st, g, a);
-  if (epi == 1) return launch_k(pdl, df_dslash_kernel<1>, grid, dim3(128), st, g, a);
-  return launch_k(pdl, df_dslash_kernel<0>, grid, dim3(128), st, g, a);
+  switch (df_tps(g)) {
+    case 4: return launch_df_tps<4>(g, a, S, epi, st, pdl);
+    case 2: return launch_df_tps<2>(g, a, S, epi, st, pdl);
+    default: return launch_df_tps<1>(g, a, S, epi, st, pdl);
+  }
 }
 
 cudaError_t launch_df_dslash(const Geom& g, const DfArgs& a, int epi, cudaStream_t st, bool pdl) {
