@@ -14,6 +14,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "internal.h"
 
 namespace lqcd {
@@ -60,16 +61,20 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
+// s + a b as four multiply-adds (GB300's FP64 pipe runs 2 per clock and SM: every operation saved counts)
+__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 s) {
+  return make_double2(fma(-a.y, b.y, fma(a.x, b.x, s.x)), fma(a.y, b.x, fma(a.x, b.y, s.y)));
+}
+
 __device__ __forceinline__ M3 mm(const M3& a, const M3& b) {  // a b
   M3 c;
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      double2 s = make_double2(0, 0);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) s = cadd(s, cmul(a.e[r * 3 + k], b.e[k * 3 + q]));
-      c.e[r * 3 + q] = s;
+      double2 s = cmul(a.e[r * 3], b.e[q]);
+      s = cfma(a.e[r * 3 + 1], b.e[3 + q], s);
+      c.e[r * 3 + q] = cfma(a.e[r * 3 + 2], b.e[6 + q], s);
     }
   return c;
 }
@@ -132,14 +137,9 @@ __global__ void __launch_bounds__(128) plaquette_kernel(Geom g, const double2* _
   }
 }
 
-// F[l][mu][a] += beta-scaled gauge force components tr(lambda^a F_g)
-__global__ void __launch_bounds__(128) gauge_force_kernel(Geom g, const double2* __restrict__ U, double beta,
-                                                          double* __restrict__ F) {
-  const int V = 2 * g.vh;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 4LL * V) return;
-  const int l = (int)(t >> 2), mu = (int)(t & 3);
-  Site s = site_at(g, l);
+// W = U_mu(x) A_mu(x), A the sum of the six staples, from the canonical links in FP64.
+static __device__ __noinline__ M3 link_times_staples(Geom g, const double2* __restrict__ U, Site s, int mu) {
+  const int l = s.l;
   const int xpmu = neighbour_addr(g, neighbour_fwd(g, s, mu));
   Site sp = site_at(g, xpmu);
   M3 A;
@@ -158,15 +158,130 @@ __global__ void __launch_bounds__(128) gauge_force_kernel(Geom g, const double2*
     add_to(A, up);
     add_to(A, dn);
   }
-  M3 W = mm(ldm(U + ((size_t)l * 4 + mu) * 9), A);
+  return mm(ldm(U + ((size_t)l * 4 + mu) * 9), A);
+}
+
+// The same products in fixed point (fixpoint.h), from the digits of 1/2 eta bc U.  A matrix is (re.h, re.l,
+// im.h, im.l) per entry, F = H 2^28 + L with L >= 0 here; a product's entries are 64-bit sums in units of 2^56 of
+// the product of the factors' units, whose digits (fix_split) are the next product's factor:
+//   folded links in units of 2^-57, entries <= 1/2;   U U in 2^-58, <= 1/4;   U U U in 2^-59, <= 1/8;
+//   the six staples' sum, divided by 4, in 2^-57, <= 3/4;   U A in 2^-58, <= 3/8.
+// The H H sums stay below 6 2^28 2^28.6 = 2^59.2, the H L sums below 6 (2^28 2^28 + 2^28 2^28.6) = 2^60; each product
+// drops and rounds less than 8 units, 2^-55 of 1/4.
+struct FixSum3 {
+  int64_t re[9], im[9];
+};
+
+// op(A) op(B), op the adjoint where AD, BD
+template <bool AD, bool BD>
+__device__ __forceinline__ FixSum3 fix_mm(const FixLink& A, const FixLink& B) {
+  FixSum3 o;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      // re = sum ar br - (+-) ai bi: the imaginary products go to accumulators of their own, so that the signs
+      // of the adjoints cost nothing
+      int64_t h1 = 0, x1 = 0, h2 = 0, x2 = 0, h3 = 0, x3 = 0, h4 = 0, x4 = 0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int4 a = A.e[AD ? 3 * k + r : 3 * r + k], b = B.e[BD ? 3 * q + k : 3 * k + q];
+        fix_mac(h1, x1, a.x, a.y, Fix2{b.x, b.y});
+        fix_mac(h2, x2, a.z, a.w, Fix2{b.z, b.w});
+        fix_mac(h3, x3, a.x, a.y, Fix2{b.z, b.w});
+        fix_mac(h4, x4, a.z, a.w, Fix2{b.x, b.y});
+      }
+      const int64_t half = 1 << (kFixLow - 1);
+      // (ar +- i ai)(br +- i bi): re = ar br - s ai bi with s = -1 where one factor is conjugated
+      const int64_t rh = AD != BD ? h1 + h2 : h1 - h2, rx = AD != BD ? x1 + x2 : x1 - x2;
+      const int64_t ih = (BD ? -h3 : h3) + (AD ? -h4 : h4), ix = (BD ? -x3 : x3) + (AD ? -x4 : x4);
+      o.re[3 * r + q] = rh + ((rx + half) >> kFixLow);
+      o.im[3 * r + q] = ih + ((ix + half) >> kFixLow);
+    }
+  }
+  return o;
+}
+
+__device__ __forceinline__ FixLink fix_split(const FixSum3& s, int shift) {  // digits of s / 2^shift
+  FixLink o;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int64_t re = s.re[j] >> shift, im = s.im[j] >> shift;
+    o.e[j] = make_int4((int)(re >> kFixLow), (int)re & ((1 << kFixLow) - 1), (int)(im >> kFixLow),
+                       (int)im & ((1 << kFixLow) - 1));
+  }
+  return o;
+}
+
+// F[l][mu][a] += beta-scaled gauge force components tr(lambda^a F_g); block: 32 sites of one parity, one direction
+// per warp.  The 13 matrix products of a link in FP64 take 1404 multiply-adds, 702 clocks of the SM's FP64 pipe; in
+// fixed point 4212 integer ones, 66 clocks, and about as much again for digits and addresses: 24^3 x 6 (331 776
+// links) 1865 -> 320 us.  Links outside the format, or no digits (Ufix null): FP64.
+__global__ void __launch_bounds__(128, 2) gauge_force_kernel(Geom g, const double2* __restrict__ U,
+                                                             const int4* __restrict__ Ufix, double beta,
+                                                             double* __restrict__ F) {
+  const int vh = g.vh;
+  const int nb = (vh + 31) / 32;
+  const int p = (int)blockIdx.x >= nb ? 1 : 0;
+  const int i = ((int)blockIdx.x - p * nb) * 32 + (threadIdx.x & 31), mu = threadIdx.x >> 5;
+  if (i >= vh) return;
+  const Site s = site_of(g, p, i);
+  double Wre[9], Wim[9];
+  bool ok = Ufix != nullptr;
+  if (ok) {
+    const uint64_t pol = policy_evict_last();  // every link is read by the 18 staples it is in
+    const int xpmu = neighbour_addr(g, neighbour_fwd(g, s, mu));
+    const Site sp = site_at(g, xpmu);
+    auto link = [&](int parity, int dir, int l) {
+      const FixLink L = load_link_fix(Ufix, parity, dir, l >> 1, vh, pol);
+      ok = ok && L.e[0].x != kFixBadLink;
+      return L;
+    };
+    FixSum3 A;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) A.re[j] = A.im[j] = 2;  // rounds the division by 4 below
+#pragma unroll 1
+    for (int m = 1; m < 4; ++m) {
+      const int nu = (mu + m) & 3;
+      const int xpnu = neighbour_addr(g, neighbour_fwd(g, s, nu));
+      const int xmnu = neighbour_addr(g, neighbour_bwd(g, s, nu));
+      const int xpmu_mnu = neighbour_addr(g, neighbour_bwd(g, sp, nu));
+      const FixLink up2 = fix_split(fix_mm<false, true>(link(1 - p, nu, xpmu), link(1 - p, mu, xpnu)), 0);
+      const FixSum3 up = fix_mm<false, true>(up2, link(p, nu, s.l));
+      // (U_mu(x-nu) U_nu(x+mu-nu))^+ U_nu(x-nu)
+      const FixLink dn2 = fix_split(fix_mm<false, false>(link(1 - p, mu, xmnu), link(p, nu, xpmu_mnu)), 0);
+      const FixSum3 dn = fix_mm<true, false>(dn2, link(1 - p, nu, xmnu));
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        A.re[j] += up.re[j] + dn.re[j];
+        A.im[j] += up.im[j] + dn.im[j];
+      }
+    }
+    const FixSum3 W = fix_mm<false, false>(link(p, mu, s.l), fix_split(A, 2));
+    // the links' factors 1/2 and eta bc: 1/16, and the staggered signs around a plaquette multiply to -1
+    const double sc = -16.0 * 0x1p-58;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      Wre[j] = (double)(long long)W.re[j] * sc;
+      Wim[j] = (double)(long long)W.im[j] * sc;
+    }
+  }
+  if (!ok) {
+    const M3 W = link_times_staples(g, U, s, mu);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      Wre[j] = W.e[j].x;
+      Wim[j] = W.e[j].y;
+    }
+  }
   // F = -(i beta/12)(W - W^+): F_rc = -(i beta/12)(W_rc - conj(W_cr)) = (beta/12)(dim + ... )
   double Fre[9], Fim[9];
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      double dre = W.e[r * 3 + c].x - W.e[c * 3 + r].x;
-      double dim = W.e[r * 3 + c].y + W.e[c * 3 + r].y;
+      double dre = Wre[r * 3 + c] - Wre[c * 3 + r];
+      double dim = Wim[r * 3 + c] + Wim[c * 3 + r];
       // -(i b)(dre + i dim) = b dim - i b dre
       Fre[r * 3 + c] = beta / 12.0 * dim;
       Fim[r * 3 + c] = -beta / 12.0 * dre;
@@ -175,7 +290,7 @@ __global__ void __launch_bounds__(128) gauge_force_kernel(Geom g, const double2*
   Fre[0] -= tr3;
   Fre[4] -= tr3;
   Fre[8] -= tr3;
-  double* o = F + ((size_t)l * 4 + mu) * 8;
+  double* o = F + ((size_t)s.l * 4 + mu) * 8;
   const double inv_sqrt3 = 0.57735026918962576451;
   o[0] += 2.0 * Fre[1];
   o[1] += -2.0 * Fim[1];
@@ -193,53 +308,81 @@ __global__ void kick_kernel(long long n, double* __restrict__ P, const double* _
   if (i < n) P[i] -= c * F[i];
 }
 
-// U <- exp(i h P) U, P = sum p^a lambda^a / 2, then SU(3) projection (rows 0, 1 Gram-Schmidt, row 2 = conj(r0 x r1))
+// U <- exp(i h P) U, P = sum p^a lambda^a / 2, then SU(3) projection (rows 0, 1 Gram-Schmidt, row 2 = conj(r0 x r1)).
+// Bound by the FP64 pipe: about 500 operations a link, 262 us at 24^3 x 6 (331 776 links; 17 us of memory traffic). A
+// Taylor series of matrix products to order 16, as before, takes 3500 operations and 2276 us.
 __global__ void __launch_bounds__(128) link_update_kernel(long long nlinks, double2* __restrict__ U,
                                                           const double* __restrict__ P, double h) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nlinks) return;
   const double* p = P + t * 8;
   const double inv_sqrt3 = 0.57735026918962576451;
-  // X = i h P, P Hermitian from Gell-Mann components
-  double2 Pm[9];
-  Pm[0] = make_double2(0.5 * (p[2] + p[7] * inv_sqrt3), 0);
-  Pm[4] = make_double2(0.5 * (-p[2] + p[7] * inv_sqrt3), 0);
-  Pm[8] = make_double2(-p[7] * inv_sqrt3, 0);
-  Pm[1] = make_double2(0.5 * p[0], -0.5 * p[1]);
-  Pm[3] = make_double2(0.5 * p[0], 0.5 * p[1]);
-  Pm[2] = make_double2(0.5 * p[3], -0.5 * p[4]);
-  Pm[6] = make_double2(0.5 * p[3], 0.5 * p[4]);
-  Pm[5] = make_double2(0.5 * p[5], -0.5 * p[6]);
-  Pm[7] = make_double2(0.5 * p[5], 0.5 * p[6]);
-  M3 X;
-  double nrm = 0.0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    X.e[i] = make_double2(-h * Pm[i].y, h * Pm[i].x);  // i h P
-    nrm += X.e[i].x * X.e[i].x + X.e[i].y * X.e[i].y;
-  }
-  // scaling and squaring: |X / 2^k|_F <= 1/4, Taylor to order 16
-  nrm = sqrt(nrm);
+  // Q = h P, Hermitian and traceless: diagonal qd, off-diagonal q01, q02, q12 (q_cr = conj(q_rc))
+  double qd[3] = {0.5 * h * (p[2] + p[7] * inv_sqrt3), 0.5 * h * (-p[2] + p[7] * inv_sqrt3), -h * p[7] * inv_sqrt3};
+  double2 q01 = make_double2(0.5 * h * p[0], -0.5 * h * p[1]);
+  double2 q02 = make_double2(0.5 * h * p[3], -0.5 * h * p[4]);
+  double2 q12 = make_double2(0.5 * h * p[5], -0.5 * h * p[6]);
+  double n01 = q01.x * q01.x + q01.y * q01.y, n02 = q02.x * q02.x + q02.y * q02.y, n12 = q12.x * q12.x + q12.y * q12.y;
+  // scaling and squaring: |Q / 2^k|_F <= 1/4
+  double nrm = sqrt(qd[0] * qd[0] + qd[1] * qd[1] + qd[2] * qd[2] + 2.0 * (n01 + n02 + n12));
   int k = 0;
   while (nrm > 0.25 && k < 30) {
     nrm *= 0.5;
     ++k;
   }
-  const double sc = ldexp(1.0, -k);
+  if (k > 0) {
+    const double sc = ldexp(1.0, -k), sc2 = sc * sc;
+    for (int c = 0; c < 3; ++c) qd[c] *= sc;
+    q01 = make_double2(q01.x * sc, q01.y * sc);
+    q02 = make_double2(q02.x * sc, q02.y * sc);
+    q12 = make_double2(q12.x * sc, q12.y * sc);
+    n01 *= sc2;
+    n02 *= sc2;
+    n12 *= sc2;
+  }
+  // S = Q^2: diagonal s, off-diagonal s01 = (qd0 + qd1) q01 + q02 conj(q12), ...
+  const double s0 = qd[0] * qd[0] + n01 + n02, s1 = qd[1] * qd[1] + n01 + n12, s2 = qd[2] * qd[2] + n02 + n12;
+  const double2 s01 = cfma(q02, make_double2(q12.x, -q12.y), make_double2((qd[0] + qd[1]) * q01.x, (qd[0] + qd[1]) * q01.y));
+  const double2 s02 = cfma(q01, q12, make_double2((qd[0] + qd[2]) * q02.x, (qd[0] + qd[2]) * q02.y));
+  const double2 s12 = cfma(make_double2(q01.x, -q01.y), q02, make_double2((qd[1] + qd[2]) * q12.x, (qd[1] + qd[2]) * q12.y));
+  // The Taylor series in the basis 1, Q, Q^2: by the Cayley-Hamilton theorem Q^3 = c1 Q + c0 with c1 = tr Q^2 / 2,
+  // c0 = det Q, so Q^n / n! = A + B Q + D Q^2 with real coefficients that follow from those of n - 1; exp(i Q) takes
+  // them with i^n.  Order 13: |Q|^14 / 14! < 2^-64 for |Q| <= 1/4.
+  const double c1 = 0.5 * (s0 + s1 + s2);
+  const double2 q0112 = cmul(q01, q12);  // c0 = qd0 qd1 qd2 + 2 Re(q01 q12 conj(q02)) - qd0 n12 - qd1 n02 - qd2 n01
+  const double c0 = qd[0] * (qd[1] * qd[2] - n12) - qd[1] * n02 - qd[2] * n01 + 2.0 * (q0112.x * q02.x + q0112.y * q02.y);
+  double A = 0.0, B = 1.0, D = 0.0;                                       // n = 1
+  double f0[2] = {1.0, 0.0}, f1[2] = {0.0, 1.0}, f2[2] = {0.0, 0.0};  // real, imaginary: n = 0 and 1
 #pragma unroll
-  for (int i = 0; i < 9; ++i) X.e[i] = make_double2(X.e[i].x * sc, X.e[i].y * sc);
-  M3 E, term;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) E.e[i] = term.e[i] = make_double2((i % 4 == 0) ? 1.0 : 0.0, 0.0);
-  for (int n = 1; n <= 16; ++n) {
-    term = mm(term, X);
-    const double inv = 1.0 / n;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      term.e[i] = make_double2(term.e[i].x * inv, term.e[i].y * inv);
-      E.e[i] = cadd(E.e[i], term.e[i]);
+  for (int n = 2; n <= 13; ++n) {
+    const double inv = 1.0 / n, Dn = D * inv;
+    const double An = c0 * Dn, Bn = fma(A, inv, c1 * Dn);
+    D = B * inv;
+    A = An;
+    B = Bn;
+    if (n & 2) {  // i^n = -1, -i
+      f0[n & 1] -= A;
+      f1[n & 1] -= B;
+      f2[n & 1] -= D;
+    } else {
+      f0[n & 1] += A;
+      f1[n & 1] += B;
+      f2[n & 1] += D;
     }
   }
+  M3 E;
+  const double2 g1 = make_double2(f1[0], f1[1]), g2 = make_double2(f2[0], f2[1]);
+  auto diag = [&](double q, double s) { return make_double2(f0[0] + g1.x * q + g2.x * s, f0[1] + g1.y * q + g2.y * s); };
+  auto conj2 = [](double2 z) { return make_double2(z.x, -z.y); };
+  E.e[0] = diag(qd[0], s0);
+  E.e[4] = diag(qd[1], s1);
+  E.e[8] = diag(qd[2], s2);
+  E.e[1] = cfma(g1, q01, cmul(g2, s01));
+  E.e[3] = cfma(g1, conj2(q01), cmul(g2, conj2(s01)));
+  E.e[2] = cfma(g1, q02, cmul(g2, s02));
+  E.e[6] = cfma(g1, conj2(q02), cmul(g2, conj2(s02)));
+  E.e[5] = cfma(g1, q12, cmul(g2, s12));
+  E.e[7] = cfma(g1, conj2(q12), cmul(g2, conj2(s12)));
   for (int i = 0; i < k; ++i) E = mm(E, E);
   M3 Un = mm(E, ldm(U + t * 9));
   // SU(3) projection
@@ -371,7 +514,7 @@ extern "C" int rhmc_trajectory(lqcd_ctx* ctx, const lqcd_rhmc_params* prm, doubl
                           prm->prec, &sst);
     if (r != LQCD_OK) return r;
     count(sst);
-    gauge_force_kernel<<<nbl, 128, 0, st>>>(g, tw->U, prm->beta, tw->F);
+    gauge_force_kernel<<<2 * ((g.vh + 31) / 32), 128, 0, st>>>(g, tw->U, ctx->gauge.ufix, prm->beta, tw->F);
     nl += 1;
     TJ_CUDA(cudaGetLastError());
     return LQCD_OK;
