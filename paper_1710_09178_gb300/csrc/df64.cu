@@ -337,7 +337,12 @@ __global__ void __launch_bounds__(256, 4) df_r_update_kernel(Geom g, const __gri
   const float2 rr_df = sd->rr_df;
   const int vh = g.vh;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool scalar_block = blockIdx.x == gridDim.x - 1;
+  const int nb = (vh + 255) / 256;  // then the scalar block, then a block per shift for its recurrence
+  const bool scalar_block = (int)blockIdx.x == nb;
+  if ((int)blockIdx.x > nb) {
+    if (!__syncthreads_or(skip)) window_scalars_shift<false>(sd, blockIdx.x - nb - 1);
+    return;
+  }
   const bool site = !scalar_block && i < vh;
   float2 rv[4][3];  // r hi, r lo, q hi, q lo: issued before the partials are summed
   if (site) {
@@ -428,104 +433,79 @@ __global__ void __launch_bounds__(256, 4) df_p_update_kernel(Geom g, const __gri
   }
 }
 
-// The pending window: p_k = P p_k0 + sum_i pi_i R_i;  x_k += X p_k0 + sum_i chi_i R_i, all in
-// double-FP32 (the window coefficients split from FP64 once per block).  One colour at a time
-// keeps the window's residuals (2 x kWindow float2 pairs) in registers.
-__global__ void __launch_bounds__(128) df_flush_kernel(Geom g, const __grid_constant__ PerSys<DfFlushArgs> pa) {
+// The pending window: p_k = P p_k0 + sum_i pi_i R_i;  x_k += X p_k0 + sum_i chi_i R_i, all in double-FP32.  One
+// thread per complex component, which keeps the window's residuals (2 x kWindow float2) in registers; the shifts
+// are spread over gridDim.z, with the next shift's vectors loaded while one is computed.  Bound by the compensated
+// arithmetic (44 multiply-adds of 10 operations per shift and component): 32^3x8 84 -> 66 us a window, 16^3x8 27.5 -> 11.7,
+// 4^4 22 -> 5.
+__global__ void __launch_bounds__(kFlushThreads) df_flush_kernel(int n3, const __grid_constant__ PerSys<DfFlushArgs> pa) {
   const DfFlushArgs& a = pa.s[blockIdx.y];  // system blockIdx.y
   pdl_wait();
   pdl_trigger();
   SolverDev* sd = a.sd;
   const int m = sd->m;
   if (m == 0) return;
-  __shared__ float2 cP[kMaxShifts], cX[kMaxShifts], cpi[kMaxShifts][kWindow], cchi[kMaxShifts][kWindow];
-  __shared__ int act[kMaxShifts];
-  const int n = sd->n;
+  __shared__ WindowCoefs<float2> w;
   const int first = sd->first;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    cP[t] = split64(sd->P[t]);
-    cX[t] = split64(sd->X[t]);
-    act[t] = sd->wactive[t];
-    for (int q = 0; q < kWindow; ++q) {
-      cpi[t][q] = (q < m) ? split64(sd->pi[t][q]) : make_float2(0.f, 0.f);
-      cchi[t][q] = (q < m) ? split64(sd->chi[t][q]) : make_float2(0.f, 0.f);
-    }
+  const int o = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = o < n3;
+  float2 Rh[kWindow], Rl[kWindow];
+#pragma unroll
+  for (int q = 0; q < kWindow; ++q) {
+    const float2* slot = reinterpret_cast<const float2*>(static_cast<const char*>(a.ring) + q * a.slot_bytes);
+    Rh[q] = (valid && q < m) ? slot[o] : make_float2(0.f, 0.f);
+    Rl[q] = (valid && q < m) ? slot[o + n3] : make_float2(0.f, 0.f);
   }
-  __syncthreads();
-  const int vh = g.vh;
-  const size_t n3 = 3 * (size_t)vh;
-  const uint64_t pol = policy_evict_first();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < vh) {
-    for (int c = 0; c < 3; ++c) {
-      const size_t o = (size_t)c * vh + i;
-      float2 Rh[kWindow], Rl[kWindow];
+  w.load(sd->P_df, sd->X_df, sd->pi_df, sd->chi_df, sd->wactive, sd->n, m);
+  const uint64_t pol = policy_evict_first();  // x_k is touched once per window: it must not displace the links
+  const int cnt = w.count, step = gridDim.z;
+  if (valid) {
+    float2 ph, pl, xh, xl;
+    auto fetch = [&](int j) {
+      const int k = w.list[j];
+      const float2* pk = first ? a.b_hi : a.pk[k];
+      ph = pk[o];
+      pl = first ? a.b_lo[o] : pk[o + n3];
+      xh = xl = make_float2(0.f, 0.f);
+      if (!first) {
+        xh = ld_hint(a.xk[k] + o, pol);
+        xl = ld_hint(a.xk[k] + o + n3, pol);
+      }
+    };
+    int j = blockIdx.z;
+    if (j < cnt) fetch(j);
+    for (; j < cnt; j += step) {
+      const int k = w.list[j];
+      const float2 p0h = ph, p0l = pl, x0h = xh, x0l = xl;
+      if (j + step < cnt) fetch(j + step);
+      // new p_k and the increment of x_k, real and imaginary parts
+      const float2 cP = w.P[k], cX = w.X[k];
+      float ps = 0.f, pc = 0.f, qs = 0.f, qc = 0.f, xs = 0.f, xc = 0.f, ys = 0.f, yc = 0.f;
+      df_mac(ps, pc, cP.x, cP.y, p0h.x, p0l.x);
+      df_mac(qs, qc, cP.x, cP.y, p0h.y, p0l.y);
+      df_mac(xs, xc, cX.x, cX.y, p0h.x, p0l.x);
+      df_mac(ys, yc, cX.x, cX.y, p0h.y, p0l.y);
 #pragma unroll
       for (int q = 0; q < kWindow; ++q) {
-        const float2* slot = reinterpret_cast<const float2*>(static_cast<const char*>(a.ring) + q * a.slot_bytes);
-        Rh[q] = (q < m) ? slot[o] : make_float2(0.f, 0.f);
-        Rl[q] = (q < m) ? slot[o + n3] : make_float2(0.f, 0.f);
+        if (q >= m) break;
+        const float2 pq = w.pi[k][q], cq = w.chi[k][q];
+        df_mac(ps, pc, pq.x, pq.y, Rh[q].x, Rl[q].x);
+        df_mac(qs, qc, pq.x, pq.y, Rh[q].y, Rl[q].y);
+        df_mac(xs, xc, cq.x, cq.y, Rh[q].x, Rl[q].x);
+        df_mac(ys, yc, cq.x, cq.y, Rh[q].y, Rl[q].y);
       }
-      float2 bh = make_float2(0.f, 0.f), bl = bh;
-      if (first) {
-        bh = a.b_hi[o];
-        bl = a.b_lo[o];
-      }
-      for (int k = 0; k < n; ++k) {
-        if (!act[k]) continue;
-        float2* pk = a.pk[k];
-        float2* xk = a.xk[k];
-        const float2 p0h = first ? bh : pk[o], p0l = first ? bl : pk[o + n3];
-        // new p_k and the increment of x_k, real and imaginary parts
-        float ps = 0.f, pc = 0.f, qs = 0.f, qc = 0.f, xs = 0.f, xc = 0.f, ys = 0.f, yc = 0.f;
-        df_mac(ps, pc, cP[k].x, cP[k].y, p0h.x, p0l.x);
-        df_mac(qs, qc, cP[k].x, cP[k].y, p0h.y, p0l.y);
-        df_mac(xs, xc, cX[k].x, cX[k].y, p0h.x, p0l.x);
-        df_mac(ys, yc, cX[k].x, cX[k].y, p0h.y, p0l.y);
-#pragma unroll
-        for (int q = 0; q < kWindow; ++q) {
-          if (q >= m) break;
-          const float2 pq = cpi[k][q], cq = cchi[k][q];
-          df_mac(ps, pc, pq.x, pq.y, Rh[q].x, Rl[q].x);
-          df_mac(qs, qc, pq.x, pq.y, Rh[q].y, Rl[q].y);
-          df_mac(xs, xc, cq.x, cq.y, Rh[q].x, Rl[q].x);
-          df_mac(ys, yc, cq.x, cq.y, Rh[q].y, Rl[q].y);
-        }
-        const float2 pre = df_norm(ps, pc), pim = df_norm(qs, qc);
-        pk[o] = make_float2(pre.x, pim.x);
-        pk[o + n3] = make_float2(pre.y, pim.y);
-        // x_k is touched once per window: stream it through L2 without displacing the links
-        float xrs = 0.f, xrc = 0.f, xis = 0.f, xic = 0.f;
-        if (!first) {
-          const float2 xh = ld_hint(xk + o, pol), xl = ld_hint(xk + o + n3, pol);
-          xrs = xh.x;
-          xrc = xl.x;
-          xis = xh.y;
-          xic = xl.y;
-        }
-        df_add(xrs, xrc, xs, xc);
-        df_add(xis, xic, ys, yc);
-        const float2 xre = df_norm(xrs, xrc), xim = df_norm(xis, xic);
-        st_hint(xk + o, make_float2(xre.x, xim.x), pol);
-        st_hint(xk + o + n3, make_float2(xre.y, xim.y), pol);
-      }
+      const float2 pre = df_norm(ps, pc), pim = df_norm(qs, qc);
+      a.pk[k][o] = make_float2(pre.x, pim.x);
+      a.pk[k][o + n3] = make_float2(pre.y, pim.y);
+      float xrs = x0h.x, xrc = x0l.x, xis = x0h.y, xic = x0l.y;
+      df_add(xrs, xrc, xs, xc);
+      df_add(xis, xic, ys, yc);
+      const float2 xre = df_norm(xrs, xrc), xim = df_norm(xis, xic);
+      st_hint(a.xk[k] + o, make_float2(xre.x, xim.x), pol);
+      st_hint(a.xk[k] + o + n3, make_float2(xre.y, xim.y), pol);
     }
   }
-  if (publish_partial(a.partials, a.ticket, 0.0)) {
-    __threadfence();
-    const int t = threadIdx.x;
-    if (t == 0) *a.ticket = 0u;
-    if (t < n) {
-      sd->P[t] = 1.0;
-      sd->X[t] = 0.0;
-      sd->wactive[t] = sd->active[t];
-    }
-    if (t == 0) {
-      advance_window_scalars(sd, m);
-      sd->m = 0;
-      sd->first = 0;
-    }
-  }
+  close_window(sd, m, a.ticket);
 }
 
 // (hi, lo) vectors -> FP64 (x = hi + lo, exact), one thread per complex component
@@ -543,9 +523,9 @@ cudaError_t launch_df_init(const Geom& g, const double2* b64, void* r, void* p, 
   return cudaGetLastError();
 }
 
-// the update kernels: one block per 256 sites plus the scalar block, per system
-cudaError_t launch_df_r_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S, cudaStream_t st, bool pdl) {
-  return launch_k(pdl, df_r_update_kernel, dim3((g.vh + 255) / 256 + 1, S), dim3(256), st, g, a);
+// the update kernels: one block per 256 sites plus the scalar block
+cudaError_t launch_df_r_update(const Geom& g, const PerSys<DfUpdArgs>& a, int n, int S, cudaStream_t st, bool pdl) {
+  return launch_k(pdl, df_r_update_kernel, dim3((g.vh + 255) / 256 + 1 + n, S), dim3(256), st, g, a);
 }
 
 cudaError_t launch_df_p_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S, cudaStream_t st, bool pdl) {
@@ -553,7 +533,8 @@ cudaError_t launch_df_p_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S,
 }
 
 cudaError_t launch_df_flush(const Geom& g, const PerSys<DfFlushArgs>& a, int S, cudaStream_t st, bool pdl) {
-  return launch_k(pdl, df_flush_kernel, dim3((g.vh + 127) / 128, S), dim3(128), st, g, a);
+  const int n3 = 3 * g.vh;
+  return launch_k(pdl, df_flush_kernel, flush_grid(n3, S), dim3(kFlushThreads), st, n3, a);
 }
 
 cudaError_t launch_df_to_fp64(const Geom& g, const void* v, double2* x, cudaStream_t st) {

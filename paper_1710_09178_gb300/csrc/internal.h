@@ -72,14 +72,17 @@ struct SolverDev {
   unsigned ticket[4];
   double s[kMaxShifts];  // sigma_k - sigma_0
   double zeta[kMaxShifts], zeta_prev[kMaxShifts];
-  // base scalars of the pending window's iterations (alpha_j, beta_j, |r_j+1|^2): the per-shift
-  // recurrences are replayed from them once per window (window_scalars_kernel)
+  // base scalars of the pending window's iterations (alpha_j, beta_j, |r_j+1|^2), from which the per-shift
+  // recurrences follow (window_scalars_shift), and how many iterations each shift's have taken
+  int wdone[kMaxShifts];
   double alpha_h[kWindow], beta_h[kWindow], rr_h[kWindow];
   int active[kMaxShifts];   // shift still iterating
   int wactive[kMaxShifts];  // shift takes part in the pending window
   // pending window: p_k = P p_k0 + sum_i pi_i R_i,  x_k = x_k0 + X p_k0 + sum_i chi_i R_i
   double P[kMaxShifts], X[kMaxShifts];
   double pi[kMaxShifts][kWindow], chi[kMaxShifts][kWindow];
+  // the same as (hi, lo) FP32 pairs (hi alone: rounded to FP32) for the window update
+  float2 P_df[kMaxShifts], X_df[kMaxShifts], pi_df[kMaxShifts][kWindow], chi_df[kMaxShifts][kWindow];
   double scal[kMaxShifts + 4];  // reduction results of auxiliary kernels
 };
 
@@ -254,7 +257,6 @@ struct DfFlushArgs {
   const float2* b_hi;  // the source as (hi, lo): p_k0 of the first window
   const float2* b_lo;
   SolverDev* sd;
-  double* partials;
   unsigned* ticket;
 };
 struct InitParams;
@@ -265,7 +267,7 @@ cudaError_t launch_df_dslash(const Geom& g, const DfArgs& a, int epi, cudaStream
 cudaError_t launch_df_dslash_multi(const Geom& g, const PerSys<DfArgs>& a, int S, int epi, cudaStream_t st, bool pdl);
 cudaError_t launch_df_init(const Geom& g, const double2* b64, void* r, void* p, SolverDev* sd, const InitParams& ip,
                            double* partials, unsigned* ticket, cudaStream_t st);
-cudaError_t launch_df_r_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S, cudaStream_t st, bool pdl);
+cudaError_t launch_df_r_update(const Geom& g, const PerSys<DfUpdArgs>& a, int n, int S, cudaStream_t st, bool pdl);
 cudaError_t launch_df_p_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S, cudaStream_t st, bool pdl);
 int df_dslash_grid_blocks(const Geom& g);  // blocks (= partials) of one double-FP32 Dslash launch
 cudaError_t launch_df_flush(const Geom& g, const PerSys<DfFlushArgs>& a, int S, cudaStream_t st, bool pdl);

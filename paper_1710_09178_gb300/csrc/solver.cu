@@ -141,7 +141,12 @@ __global__ void __launch_bounds__(256, 4) r_update_kernel(Geom g, const __grid_c
   const double rr = sd->rr;
   const float2 rr_df = sd->rr_df;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool scalar_block = blockIdx.x == gridDim.x - 1;
+  const int nb = (g.vh + 255) / 256;  // then the scalar block, then a block per shift for its recurrence
+  const bool scalar_block = (int)blockIdx.x == nb;
+  if ((int)blockIdx.x > nb) {
+    if (!__syncthreads_or(skip)) window_scalars_shift<false>(sd, blockIdx.x - nb - 1);
+    return;
+  }
   const bool site = !scalar_block && i < g.vh;
   Vec3<T> r, q;
   if (site) {
@@ -233,34 +238,115 @@ struct FlushArgs {
   double2* xk[kMaxShifts];
   const double2* b64;
   SolverDev* sd;
-  double* partials;
   unsigned* ticket;
 };
 
 // Apply the pending window: p_k = P p_k0 + sum_i pi_i R_i;  x_k += X p_k0 + sum_i chi_i R_i.
-// At the first window of a solve p_k0 = b and x_k0 = 0 (nothing is read).
-template <typename T, int SF, bool XDF>
-__global__ void __launch_bounds__(128) flush_kernel(Geom g, const __grid_constant__ PerSys<FlushArgs> pa) {
+// At the first window of a solve p_k0 = b and x_k0 = 0 (nothing is read).  One thread per complex component
+// keeps the window's residuals in registers; the shifts are spread over gridDim.z, with the next shift's vectors
+// loaded while one is computed.  FP32: bound by HBM on large lattices (32^3x8: 36 -> 25 us a window with x_k as pairs),
+// by latency on small ones (16^3x8 11 -> 7 us; one thread per site walked 3 colours x all shifts before).  FP64: by the
+// FP64 pipe (16^3x8 31 -> 29 us).  XDF: x_k as (hi, lo) FP32 pairs, else FP64.
+template <typename T, bool XDF>
+__global__ void __launch_bounds__(kFlushThreads) flush_kernel(int n3, const __grid_constant__ PerSys<FlushArgs> pa) {
+  typedef typename KTraits<T>::V2 V2;
   const FlushArgs& a = pa.s[blockIdx.y];  // system blockIdx.y
   SolverDev* sd = a.sd;
   pdl_wait();
   pdl_trigger();
   const int m = sd->m;
   if (m == 0) return;  // nothing pending
-  __shared__ T cP[kMaxShifts], cX[kMaxShifts], cpi[kMaxShifts][kWindow], cchi[kMaxShifts][kWindow];
-  __shared__ int act[kMaxShifts];
-  const int n = sd->n;
+  __shared__ WindowCoefs<T> w;
   const int first = sd->first;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    cP[t] = (T)sd->P[t];
-    cX[t] = (T)sd->X[t];
-    act[t] = sd->wactive[t];
-    for (int s = 0; s < kWindow; ++s) {
-      cpi[t][s] = (s < m) ? (T)sd->pi[t][s] : (T)0;
-      cchi[t][s] = (s < m) ? (T)sd->chi[t][s] : (T)0;
+  const int o = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = o < n3;
+  V2 R[kWindow];
+#pragma unroll
+  for (int s = 0; s < kWindow; ++s) {
+    R[s].x = R[s].y = 0;
+    if (valid && s < m) R[s] = reinterpret_cast<const V2*>(static_cast<const char*>(a.ring) + s * a.slot_bytes)[o];
+  }
+  if constexpr (sizeof(T) == 4) w.load(sd->P_df, sd->X_df, sd->pi_df, sd->chi_df, sd->wactive, sd->n, m);
+  else w.load(sd->P, sd->X, sd->pi, sd->chi, sd->wactive, sd->n, m);
+  const uint64_t pol = policy_evict_first();  // x_k is touched once per window: it must not displace the links
+  const int cnt = w.count, step = gridDim.z;
+  if (valid) {
+    V2 pn;
+    float2 xh, xl;
+    double2 xd;
+    auto fetch = [&](int j) {
+      const int k = w.list[j];
+      if (first) {
+        const double2 b = a.b64[o];
+        pn.x = (T)b.x;
+        pn.y = (T)b.y;
+        xh = xl = make_float2(0.f, 0.f);
+        xd = make_double2(0.0, 0.0);
+      } else {
+        pn = static_cast<const V2*>(a.pk[k])[o];
+        if constexpr (XDF) {
+          xh = ld_hint(reinterpret_cast<const float2*>(a.xk[k]) + o, pol);
+          xl = ld_hint(reinterpret_cast<const float2*>(a.xk[k]) + o + n3, pol);
+        } else {
+          xd = ld_hint(a.xk[k] + o, pol);
+        }
+      }
+    };
+    int j = blockIdx.z;
+    if (j < cnt) fetch(j);
+    for (; j < cnt; j += step) {
+      const int k = w.list[j];
+      const V2 p0 = pn;
+      const float2 x0h = xh, x0l = xl;
+      const double2 x0 = xd;
+      if (j + step < cnt) fetch(j + step);
+      const T P = w.P[k], X = w.X[k];
+      V2 np, dx;
+      np.x = P * p0.x;
+      np.y = P * p0.y;
+      dx.x = X * p0.x;
+      dx.y = X * p0.y;
+#pragma unroll
+      for (int s = 0; s < kWindow; ++s) {
+        const T pis = w.pi[k][s], chs = w.chi[k][s];
+        np.x = fma(pis, R[s].x, np.x);
+        np.y = fma(pis, R[s].y, np.y);
+        dx.x = fma(chs, R[s].x, dx.x);
+        dx.y = fma(chs, R[s].y, dx.y);
+      }
+      static_cast<V2*>(a.pk[k])[o] = np;
+      if constexpr (XDF) {
+        // (hi, lo) FP32 pairs: the window's increment added with TwoSum, no FP64 instruction
+        float2* xp = reinterpret_cast<float2*>(a.xk[k]);
+        float rs = x0h.x, rc = x0l.x, is = x0h.y, ic = x0l.y;
+        df_add(rs, rc, (float)dx.x, 0.f);
+        df_add(is, ic, (float)dx.y, 0.f);
+        const float2 re = df_norm(rs, rc), im = df_norm(is, ic);
+        st_hint(xp + o, make_float2(re.x, im.x), pol);
+        st_hint(xp + o + n3, make_float2(re.y, im.y), pol);
+      } else {
+        st_hint(a.xk[k] + o, make_double2(x0.x + (double)dx.x, x0.y + (double)dx.y), pol);
+      }
     }
   }
-  __syncthreads();
+  close_window(sd, m, a.ticket);
+}
+
+// The same with the shift vectors in 16-bit fixed point: one thread per site (a record holds all three colours and
+// their scale).
+template <bool XDF>
+__global__ void __launch_bounds__(kFlushThreads) flush16_kernel(Geom g, const __grid_constant__ PerSys<FlushArgs> pa) {
+  const FlushArgs& a = pa.s[blockIdx.y];  // system blockIdx.y
+  SolverDev* sd = a.sd;
+  pdl_wait();
+  pdl_trigger();
+  const int m = sd->m;
+  if (m == 0) return;  // nothing pending
+  typedef float T;
+  constexpr int SF = kS16;
+  __shared__ WindowCoefs<T> w;
+  const int first = sd->first;
+  w.load(sd->P_df, sd->X_df, sd->pi_df, sd->chi_df, sd->wactive, sd->n, m);
   const int vh = g.vh;
   const uint64_t pol = policy_evict_first();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -271,11 +357,11 @@ __global__ void __launch_bounds__(128) flush_kernel(Geom g, const __grid_constan
       R[s] = (s < m) ? load_s<SF, T>(static_cast<const char*>(a.ring) + s * a.slot_bytes, i, vh) : vzero<T>();
     Vec3<T> b0 = vzero<T>();
     if (first) b0 = to_t<T>(load_vec(a.b64, i, vh));
-    for (int k = 0; k < n; ++k) {
-      if (!act[k]) continue;
+    for (int j = blockIdx.z; j < w.count; j += gridDim.z) {
+      const int k = w.list[j];
       Vec3<T> p0 = first ? b0 : load_s<SF, T>(a.pk[k], i, vh);
       Vec3<T> np, dx;
-      const T P = cP[k], X = cX[k];
+      const T P = w.P[k], X = w.X[k];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         np.c[c] = cmake(P * p0.c[c].re, P * p0.c[c].im);
@@ -283,7 +369,7 @@ __global__ void __launch_bounds__(128) flush_kernel(Geom g, const __grid_constan
       }
 #pragma unroll
       for (int s = 0; s < kWindow; ++s) {
-        const T pis = cpi[k][s], chs = cchi[k][s];
+        const T pis = w.pi[k][s], chs = w.chi[k][s];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           np.c[c].re = fma(pis, R[s].c[c].re, np.c[c].re);
@@ -325,29 +411,15 @@ __global__ void __launch_bounds__(128) flush_kernel(Geom g, const __grid_constan
       }
     }
   }
-  if (publish_partial(a.partials, a.ticket, 0.0)) {
-    __threadfence();
-    int t = threadIdx.x;
-    if (t == 0) *a.ticket = 0u;
-    if (t < n) {
-      sd->P[t] = 1.0;
-      sd->X[t] = 0.0;
-      sd->wactive[t] = sd->active[t];
-    }
-    if (t == 0) {
-      advance_window_scalars(sd, m);
-      sd->m = 0;
-      sd->first = 0;
-    }
-  }
+  close_window(sd, m, a.ticket);
 }
 
-// Per-shift recurrences of the pending window, right before the window update: block (k, s) is
-// shift k of system s.
+// The per-shift recurrences that the window's r updates have not taken (its last iteration's), right before the
+// window update: block (k, s) is shift k of system s.
 __global__ void window_scalars_kernel(const __grid_constant__ PerSys<SolverDev*> sds) {
   pdl_wait();
   pdl_trigger();
-  window_scalars_shift(sds.s[blockIdx.y], blockIdx.x);
+  window_scalars_shift<true>(sds.s[blockIdx.y], blockIdx.x);
 }
 
 // Precision schedule of the mixed modes.  The error that FP32 arithmetic (links, Krylov vectors)
@@ -783,13 +855,13 @@ static DfBufs df_bufs(Workspace* w, bool phase) {
 }
 
 // the four kernels of one base iteration
-static cudaError_t enqueue_iteration_df(Launcher& L, bool phase);
+static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase);
 
-static cudaError_t enqueue_iteration(Launcher& L) {
+static cudaError_t enqueue_iteration(Launcher& L, int n) {
   Workspace* w = L.w;
   lqcd_ctx* ctx = L.ctx;
   cudaStream_t st = w->st;
-  if (w->kprec == LQCD_DF64) return enqueue_iteration_df(L, false);
+  if (w->kprec == LQCD_DF64) return enqueue_iteration_df(L, n, false);
   const int S = L.S;
   PerSys<DslashArgs> d1, d2;
   PerSys<RUpdArgs> ra;
@@ -854,10 +926,10 @@ static cudaError_t enqueue_iteration(Launcher& L) {
   }
   if (e != cudaSuccess) return e;
   const bool pr = L.next_pdl();
-  const dim3 grid(nb + 1, S);
-  if (w->kprec == LQCD_FP64) e = launch_k(pr, r_update_kernel<double, kS64>, grid, dim3(256), st, L.g, ra);
-  else if (w->sfmt == kS16) e = launch_k(pr, r_update_kernel<float, kS16>, grid, dim3(256), st, L.g, ra);
-  else e = launch_k(pr, r_update_kernel<float, kS32>, grid, dim3(256), st, L.g, ra);
+  const dim3 grid(nb + 1, S), rgrid(nb + 1 + n, S);  // one block per shift for its recurrence
+  if (w->kprec == LQCD_FP64) e = launch_k(pr, r_update_kernel<double, kS64>, rgrid, dim3(256), st, L.g, ra);
+  else if (w->sfmt == kS16) e = launch_k(pr, r_update_kernel<float, kS16>, rgrid, dim3(256), st, L.g, ra);
+  else e = launch_k(pr, r_update_kernel<float, kS32>, rgrid, dim3(256), st, L.g, ra);
   L.nlaunch += 1;
   if (e != cudaSuccess) return e;
   const bool pp = L.next_pdl();
@@ -869,7 +941,7 @@ static cudaError_t enqueue_iteration(Launcher& L) {
 
 // the four kernels of one base iteration of the double-FP32 solve (LQCD_DF64, or the double-FP32
 // phase of a mixed solve)
-static cudaError_t enqueue_iteration_df(Launcher& L, bool phase) {
+static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase) {
   Workspace* w = L.w;
   lqcd_ctx* ctx = L.ctx;
   cudaStream_t st = w->st;
@@ -923,7 +995,7 @@ static cudaError_t enqueue_iteration_df(Launcher& L, bool phase) {
   e = launch_df_dslash_multi(L.g, a, S, 1, st, L.next_pdl());
   L.nlaunch += 1;
   if (e != cudaSuccess) return e;
-  e = launch_df_r_update(L.g, u, S, st, L.next_pdl());
+  e = launch_df_r_update(L.g, u, n, S, st, L.next_pdl());
   L.nlaunch += 1;
   if (e != cudaSuccess) return e;
   e = launch_df_p_update(L.g, u, S, st, L.next_pdl());
@@ -957,7 +1029,6 @@ static cudaError_t enqueue_flush(Launcher& L, int n, bool df_phase = false) {
       f.b_hi = y->dfb_h;
       f.b_lo = y->dfb_l;
       f.sd = y->sd;
-      f.partials = y->partials;
       f.ticket = y->tickets + 2;
     }
     L.nlaunch += 1;
@@ -977,19 +1048,21 @@ static cudaError_t enqueue_flush(Launcher& L, int n, bool df_phase = false) {
     }
     f.b64 = y->b64;
     f.sd = y->sd;
-    f.partials = y->partials;
     f.ticket = y->tickets + 2;
   }
-  const dim3 grid((L.g.vh + 127) / 128, S);
+  const int n3 = 3 * L.g.vh;
   const bool pdl = L.next_pdl();
   L.nlaunch += 1;
-  if (w->sfmt == kS64) return launch_k(pdl, flush_kernel<double, kS64, false>, grid, dim3(128), w->st, L.g, fa);
+  const dim3 threads(kFlushThreads);
   if (w->sfmt == kS16) {
-    if (w->xdfmode) return launch_k(pdl, flush_kernel<float, kS16, true>, grid, dim3(128), w->st, L.g, fa);
-    return launch_k(pdl, flush_kernel<float, kS16, false>, grid, dim3(128), w->st, L.g, fa);
+    const dim3 grid = flush_grid(L.g.vh, S);
+    if (w->xdfmode) return launch_k(pdl, flush16_kernel<true>, grid, threads, w->st, L.g, fa);
+    return launch_k(pdl, flush16_kernel<false>, grid, threads, w->st, L.g, fa);
   }
-  if (w->xdfmode) return launch_k(pdl, flush_kernel<float, kS32, true>, grid, dim3(128), w->st, L.g, fa);
-  return launch_k(pdl, flush_kernel<float, kS32, false>, grid, dim3(128), w->st, L.g, fa);
+  const dim3 grid = flush_grid(n3, S);
+  if (w->sfmt == kS64) return launch_k(pdl, flush_kernel<double, false>, grid, threads, w->st, n3, fa);
+  if (w->xdfmode) return launch_k(pdl, flush_kernel<float, true>, grid, threads, w->st, n3, fa);
+  return launch_k(pdl, flush_kernel<float, false>, grid, threads, w->st, n3, fa);
 }
 
 // FP64 residual r64 = bvec - (A + sigma) x into r64, |r64|^2 into *dot (device); one system
@@ -1151,7 +1224,7 @@ static cudaError_t enqueue_df_window(Launcher& L, int n, cudaGraphConditionalHan
   const int S = L.S;
   cudaError_t e;
   for (int it = 0; it < kWindow; ++it)
-    if ((e = enqueue_iteration_df(L, true)) != cudaSuccess) return e;
+    if ((e = enqueue_iteration_df(L, n, true)) != cudaSuccess) return e;
   if ((e = enqueue_flush(L, n, true)) != cudaSuccess) return e;
   loop_ctl_df_kernel<<<1, 32, 0, w->st>>>(handle, solver_states(L), S, set_cond);
   L.nlaunch += 1;
@@ -1190,7 +1263,7 @@ static cudaError_t enqueue_batch(Launcher& L, int n, int k0, double sigma0, int 
   const int S = L.S;
   for (int wdx = 0; wdx < windows; ++wdx) {
     for (int it = 0; it < kWindow; ++it)
-      if ((e = enqueue_iteration(L)) != cudaSuccess) return e;
+      if ((e = enqueue_iteration(L, n)) != cudaSuccess) return e;
     if ((e = enqueue_flush(L, n)) != cudaSuccess) return e;
     if (use_ru && w->df) {
       // r = fl32(b - (A + sigma_0) x_0) in double-FP32 straight into the Krylov residual

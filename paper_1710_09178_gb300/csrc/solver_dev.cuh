@@ -1,6 +1,6 @@
 // solver_dev.cuh - the scalar steps of the shifted CG: the base steps run by one block right after
 // the global sum they need is known (the extra block of the r and p update kernels), and the
-// per-shift recurrences of a window, replayed once per window before the window update.
+// per-shift recurrences of a window, one iteration behind them (n extra blocks of the r update).
 //
 // Shifted CG (Section 4; ref. [mcg]): base system A + sigma_0 with sigma_0 the
 // smallest shift, s_k = sigma_k - sigma_0, residual collinearity r_k = zeta_k r.
@@ -9,7 +9,7 @@
 //   beta step (needs (r,r) new): beta = (r,r)_new/(r,r);  beta_k = beta (zeta_k'/zeta_k)^2;
 //       p_k = zeta_k' r_new + beta_k p_k;  stop shift k once zeta_k'^2 (r,r)_new <= tol^2 (b,b);
 //       and decide whether a reliable update is due at the end of the window
-// (the zeta_k parts of both steps are deferred to the window end, window_scalars_shift())
+// (the zeta_k parts of both steps follow one iteration later, window_scalars_shift())
 // The x_k and p_k updates are not applied vector by vector: they are folded into
 // the coefficients of the pending window,
 //   p_k = P p_k0 + sum_i pi_i R_i,   x_k = x_k0 + X p_k0 + sum_i chi_i R_i,
@@ -43,6 +43,7 @@ __device__ __forceinline__ void init_scalars(SolverDev* sd, const InitParams& ip
     sd->s[k] = ip.s[k];
     sd->zeta[k] = sd->zeta_prev[k] = 1.0;
     sd->active[k] = sd->wactive[k] = trivial ? 0 : 1;
+    sd->wdone[k] = 0;
     sd->P[k] = 1.0;
     sd->X[k] = 0.0;
   }
@@ -86,9 +87,7 @@ __device__ __forceinline__ void init_scalars(SolverDev* sd, const InitParams& ip
 // The base iteration needs only alpha and beta; the per-shift recurrences (zeta_k, the window
 // coefficients, the stopping tests of the shifts) depend on nothing but the sequence of alpha and
 // beta.  So the two steps below store the base scalars of the iteration and decide the base
-// stopping test, and window_scalars_shift() replays the per-shift recurrences of the whole window once,
-// before the window update, with the same operations in the same order as an iteration-by-iteration
-// evaluation.  The base shift stops last: for s_k >= 0, |zeta_k| <= 1 (zeta_k is the inverse of the
+// stopping test, and window_scalars_shift() follows with the per-shift recurrences.  The base shift stops last: for s_k >= 0, |zeta_k| <= 1 (zeta_k is the inverse of the
 // base residual polynomial at -s_k), and zeta_0 = 1 exactly, so "every shift has stopped" is "the
 // base residual has": |r_new|^2 <= tol^2 |b|^2.
 
@@ -149,11 +148,10 @@ __device__ __forceinline__ void solver_beta_step(SolverDev* sd, const PartialsRa
   sd->ru_skip = (done || !due) ? 1 : 0;
 }
 
-// Per-shift recurrences of the pending window's m iterations for shift k, replayed from alpha_h,
-// beta_h, rr_h; one warp per shift (one block per shift, so the shifts' FP64 chains run on
-// different SMs: GB300's FP64 pipe is narrow), lane i owns the window coefficients pi_i, chi_i of
-// the shift and every lane evaluates the shift's scalar chain (the same bits in every lane).
-// Iteration j (alpha = alpha_h[j], beta = beta_h[j]):
+// The per-shift recurrences of the pending window's iterations wdone[k] .. m - 1 for shift k, from alpha_h, beta_h, rr_h;
+// one warp per shift (one block per shift, so the shifts' FP64 chains run on different SMs: GB300's FP64 pipe is
+// narrow), lane i owns the window coefficients pi_i, chi_i of the shift and every lane evaluates the shift's
+// scalar chain (the same bits in every lane).  Iteration j (alpha = alpha_h[j], beta = beta_h[j]):
 //   alpha part:  den = alpha beta_prev (zeta_prev - zeta) + zeta_prev alpha_prev (1 + s_k alpha)
 //                q = zeta_prev alpha_prev / den,  zeta' = zeta q,  alpha_k = alpha q
 //                x_k += alpha_k p_k    ->  X += alpha_k P,  chi_i += alpha_k pi_i  (i < j)
@@ -161,31 +159,31 @@ __device__ __forceinline__ void solver_beta_step(SolverDev* sd, const PartialsRa
 //                p_k = zeta' r_j+1 + beta_k p_k  ->  P *= beta_k, pi_i *= beta_k (i < j), pi_j = zeta'
 //                shift k stops once zeta'^2 |r_j+1|^2 <= tol^2 |b|^2 (then takes no later residual)
 // (zeta' = zeta zeta_prev alpha_prev / den, formed as zeta q: one FP64 division.)
-// The statistics are integer atomics (the same totals in any order): the shift's active iterations
-// go to shift_iters, and a shift that stops takes itself off n_active.  alpha_prev and beta_prev are
-// read here and advanced by the window update that follows (its last block), so no block of this
-// launch sees another's write.
+// An iteration's chain takes about 0.9 us.  So n extra blocks of the r update run iteration j - 1's while the others
+// stream the residual of iteration j, and only the last one of the window is left for its end (9.4 us there
+// when all ten were).  The statistics are integer atomics (the same totals in any order): the shift's active
+// iterations go to shift_iters, and a shift that stops takes itself off n_active.  alpha_prev and beta_prev are
+// advanced by the window update that follows (its last block), so no block of this launch sees another's write.
+// END: the window's end, which also leaves the coefficients' FP32 forms for the window update.
+template <bool END>
 __device__ __forceinline__ void window_scalars_shift(SolverDev* sd, int k) {
   if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  const int n = sd->n, m = sd->m;
-  if (k >= n || !sd->active[k]) return;  // uniform: a stopped shift keeps its state
-  const double stop2 = sd->stop2;
-  double ap = sd->alpha_prev, bp = sd->beta_prev;
-  double z = sd->zeta[k], zp = sd->zeta_prev[k];
-  const double sk = sd->s[k];
-  double P = sd->P[k], X = sd->X[k];
-  double pi = 0.0, chi = 0.0;  // slot lane of the window
-  // the window's base scalars: lane j loads iteration j's, all at once (no chain of dependent loads)
-  double al = 0.0, be = 0.0, rn = 0.0;
-  if (lane < m) {
-    al = sd->alpha_h[lane];
-    be = sd->beta_h[lane];
-    rn = sd->rr_h[lane];
+  const int lane = threadIdx.x, slot = min(lane, kWindow - 1);
+  // all loads at once (no chain of dependent ones); lane j holds iteration j's base scalars and slot j
+  const int n = sd->n, m = min(sd->m, kWindow), j0 = sd->wdone[k], active = sd->active[k];
+  const double stop2 = sd->stop2, sk = sd->s[k], al = sd->alpha_h[slot], be = sd->beta_h[slot], rn = sd->rr_h[slot];
+  double ap = sd->alpha_prev, bp = sd->beta_prev, z = sd->zeta[k], zp = sd->zeta_prev[k], P = sd->P[k], X = sd->X[k];
+  double pi = sd->pi[k][slot], chi = sd->chi[k][slot];
+  // uniform: a stopped shift keeps its state (at the window's end, one that stopped within it leaves its forms)
+  if (k >= n || !(END ? sd->wactive[k] : active && j0 < m)) return;
+  if (lane >= j0) pi = chi = 0.0;
+  if (j0) {
+    ap = __shfl_sync(0xffffffffu, al, j0 - 1);
+    bp = __shfl_sync(0xffffffffu, be, j0 - 1);
   }
-  bool act = true;
+  bool act = active != 0;
   int iters = 0;
-  for (int j = 0; j < m; ++j) {
+  for (int j = j0; j < m; ++j) {
     const double alpha = __shfl_sync(0xffffffffu, al, j), beta = __shfl_sync(0xffffffffu, be, j),
                  rr_new = __shfl_sync(0xffffffffu, rn, j);
     if (act) {  // uniform over the warp
@@ -201,8 +199,6 @@ __device__ __forceinline__ void window_scalars_shift(SolverDev* sd, int k) {
       const bool stop = zn * zn * rr_new <= stop2;
       if (lane < j) pi = pi * bk;
       else if (lane == j) pi = zn;
-      else if (stop) pi = 0.0;
-      if (lane == j || (lane > j && stop)) chi = 0.0;
       zp = z;
       z = zn;
       if (stop) act = false;
@@ -210,18 +206,27 @@ __device__ __forceinline__ void window_scalars_shift(SolverDev* sd, int k) {
     ap = alpha;
     bp = beta;
   }
-  if (lane < m) {
+  if (lane < kWindow) {  // slots not reached yet: 0
     sd->pi[k][lane] = pi;
     sd->chi[k][lane] = chi;
+    if (END) {
+      sd->pi_df[k][lane] = split_hi_lo(pi);
+      sd->chi_df[k][lane] = split_hi_lo(chi);
+    }
   }
   if (lane == 0) {
     sd->zeta[k] = z;
     sd->zeta_prev[k] = zp;
     sd->P[k] = P;
     sd->X[k] = X;
+    sd->wdone[k] = m;
     sd->active[k] = act ? 1 : 0;
+    if (END) {
+      sd->P_df[k] = split_hi_lo(P);
+      sd->X_df[k] = split_hi_lo(X);
+    }
     atomicAdd(&sd->shift_iters, iters);
-    if (!act) atomicSub(&sd->n_active, 1);
+    if (active && !act) atomicSub(&sd->n_active, 1);
   }
 }
 
@@ -230,6 +235,84 @@ __device__ __forceinline__ void window_scalars_shift(SolverDev* sd, int k) {
 __device__ __forceinline__ void advance_window_scalars(SolverDev* sd, int m) {
   sd->alpha_prev = sd->alpha_h[m - 1];
   sd->beta_prev = sd->beta_h[m - 1];
+  sd->m = 0;
+  sd->first = 0;
+}
+
+// ---------------------------------------------------------------------------
+// The window update's shared parts (flush kernels).
+// ---------------------------------------------------------------------------
+constexpr int kFlushThreads = 128;
+
+// Blocks of a window update over n3 components of S systems, and the shifts' split over blockIdx.z: as many parts (up
+// to 8) as keep the grid within two blocks per SM, so that a small lattice's shifts run side by side (4^4: 22 -> 5 us
+// a double-FP32 window); every part loads the window's residuals again (four systems on 8^4: no gain from 3 parts).
+inline dim3 flush_grid(int n3, int S) {
+  const int nb = (n3 + kFlushThreads - 1) / kFlushThreads;
+  const int z = 304 / (nb * S);
+  return dim3((unsigned)nb, (unsigned)S, (unsigned)(z < 1 ? 1 : (z > 8 ? 8 : z)));
+}
+
+// The window's coefficients in shared memory (T: FP64, FP32, or (hi, lo) pairs) and the shifts that take part.
+__device__ __forceinline__ void coef_set(double& d, double v) { d = v; }
+__device__ __forceinline__ void coef_set(float& d, float2 v) { d = v.x; }
+__device__ __forceinline__ void coef_set(float2& d, float2 v) { d = v; }
+template <typename T>
+struct WindowCoefs {
+  T P[kMaxShifts], X[kMaxShifts], pi[kMaxShifts][kWindow], chi[kMaxShifts][kWindow];
+  int list[kMaxShifts], count;
+
+  // all threads of the block call; ends with a barrier
+  template <typename S>
+  __device__ __forceinline__ void load(const S* sP, const S* sX, const S (*spi)[kWindow], const S (*schi)[kWindow],
+                                       const int* wactive, int n, int m) {
+    for (int t = threadIdx.x; t < n * kWindow; t += blockDim.x) {
+      const int k = t / kWindow, q = t - k * kWindow;
+      if (q < m) {
+        coef_set(pi[k][q], spi[k][q]);
+        coef_set(chi[k][q], schi[k][q]);
+      } else {
+        pi[k][q] = chi[k][q] = T{};
+      }
+    }
+    if (threadIdx.x < 32) {
+      const int k = threadIdx.x;
+      const bool on = k < n && wactive[k];
+      if (on) {
+        coef_set(P[k], sP[k]);
+        coef_set(X[k], sX[k]);
+      }
+      const unsigned mask = __ballot_sync(0xffffffffu, on);
+      if (on) list[__popc(mask & ((1u << k) - 1))] = k;
+      if (k == 0) count = __popc(mask);
+    }
+    __syncthreads();
+  }
+};
+
+// The end of a window update (all threads of the block call): the last block of the grid's x and z opens the next
+// window.
+__device__ __forceinline__ void close_window(SolverDev* sd, int m, unsigned* ticket) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.z - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int t = threadIdx.x;
+  if (t < sd->n) {
+    sd->P[t] = 1.0;
+    sd->X[t] = 0.0;
+    sd->wactive[t] = sd->active[t];
+    sd->wdone[t] = 0;
+  }
+  if (t == 0) {
+    *ticket = 0u;
+    advance_window_scalars(sd, m);
+  }
 }
 
 }  // namespace lqcd
