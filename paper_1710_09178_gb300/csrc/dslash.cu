@@ -13,6 +13,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fix64.cuh"
@@ -226,6 +227,42 @@ struct SiteHops {
   }
 };
 
+// The same hops with every load issued at once: all links by start(), all vectors by apply().  The sums and
+// their order are those of SiteHops<LF, 1>, so the bits are too.  About 230 registers (18-real links).
+template <int LF>
+struct SiteHopsAhead {
+  int nb[8], sg[8];
+  RawLink<LF> W[8];
+
+  __device__ __forceinline__ void start(const Geom& g, const void* links, int p, int i, int, uint64_t pol) {
+    const Site s = site_of(g, p, i);
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      const int mu = h >> 1;
+      const bool fwd = (h & 1) == 0;
+      nb[h] = neighbour_half(g, fwd ? neighbour_fwd(g, s, mu) : neighbour_bwd(g, s, mu));
+      sg[h] = (LF >= kL12) ? (fwd ? link_sign_fwd(g, s, mu) : link_sign_bwd(g, s, mu)) : 1;
+      W[h] = fwd ? load_raw<LF>(links, p, mu, i, g.vh, pol) : load_raw<LF>(links, 1 - p, mu, nb[h], g.vh, pol);
+    }
+  }
+
+  __device__ __forceinline__ Vec3<float> apply(const void*, const float2* in, int, int, int, int vh, uint64_t) {
+    Vec3<float> v[8], accf = vzero<float>(), accb = vzero<float>();
+#pragma unroll
+    for (int h = 0; h < 8; ++h) v[h] = ldg_vec(in, nb[h], vh);
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      const Mat3<float> M = decode<LF>(W[h], sg[h]);
+      if ((h & 1) == 0) mv_acc(accf, M, v[h]);
+      else mdv_acc(accb, M, v[h]);
+    }
+    Vec3<float> d;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d.c[c] = cmake(accf.c[c].re - accb.c[c].re, accf.c[c].im - accb.c[c].im);
+    return d;
+  }
+};
+
 // The chunk of output sites block blockIdx.x works on.  order 0: chunk b = block b (lexicographic
 // within the parity, the order of the stored vectors); order 1: the two halves of the site range
 // interleaved, even blocks taking the first half and odd blocks the second, so that blocks that run
@@ -238,10 +275,12 @@ __device__ __forceinline__ int site_block(int order) {
   return (b & 1) ? h + (b >> 1) : (b >> 1);
 }
 
-template <int LF, int TPS, int EPI>
-__global__ void __launch_bounds__(128, 7) dslash_kernel(Geom g, KArgs k) {
+// AHEAD (TPS = 1): small lattices, whose launches are all latency (launch_tps).
+template <int LF, int TPS, int EPI, bool AHEAD = false>
+__global__ void __launch_bounds__(128, AHEAD ? 1 : 7) dslash_kernel(Geom g, KArgs k) {
   typedef float T;
   typedef float2 V2;
+  typedef typename std::conditional<AHEAD, SiteHopsAhead<LF>, SiteHops<LF, TPS>>::type Hops;
   const int vh = g.vh;
   const int gt = site_block(k.order) * blockDim.x + threadIdx.x;
   const int i = gt / TPS;
@@ -250,7 +289,7 @@ __global__ void __launch_bounds__(128, 7) dslash_kernel(Geom g, KArgs k) {
   const int p = k.out_parity;
   const V2* in = static_cast<const V2*>(k.in);
   const uint64_t pol = policy_evict_last();
-  SiteHops<LF, TPS> hops;
+  Hops hops;
   // links are never written by the kernels of a solve: the first one is fetched before the wait
   if (valid) hops.start(g, k.links, p, i, sub, pol);
   pdl_wait();
@@ -532,6 +571,18 @@ template <int LF, int TPS>
 static cudaError_t launch_tps(const Geom& g, const KArgs& k, Epi epi, cudaStream_t st, int bs, bool pdl) {
   long long threads = (long long)g.vh * TPS;
   unsigned nb = (unsigned)((threads + bs - 1) / bs);
+  // At most one block per SM: all loads at once.  Half Dslash per graph launch, 18-real links: 8^4 2.32 -> 1.98 us, 16^3x8
+  // (128 blocks) 2.68 -> 2.38; with more blocks the other warps hide the latency better: 16^3x10 (160) 2.64 and 2.83,
+  // 20^3x8 (250) 3.07 and 3.20, 24^3x6 (324) 3.37 and 4.72.
+  if constexpr (TPS == 1) {
+    if (nb <= kSMs) {
+      switch (epi) {
+        case Epi::Plain: return launch_k(pdl, dslash_kernel<LF, 1, 0, true>, dim3(nb), dim3(bs), st, g, k);
+        case Epi::AApply: return launch_k(pdl, dslash_kernel<LF, 1, 1, true>, dim3(nb), dim3(bs), st, g, k);
+        default: return launch_k(pdl, dslash_kernel<LF, 1, 2, true>, dim3(nb), dim3(bs), st, g, k);
+      }
+    }
+  }
   switch (epi) {
     case Epi::Plain: return launch_k(pdl, dslash_kernel<LF, TPS, 0>, dim3(nb), dim3(bs), st, g, k);
     case Epi::AApply: return launch_k(pdl, dslash_kernel<LF, TPS, 1>, dim3(nb), dim3(bs), st, g, k);
