@@ -750,7 +750,7 @@ __device__ __forceinline__ double warp_sum_df(const float2* p, int n) {
 // any block size (a multiple of 64) that sum the same partials get the same bits.  Thread t takes
 // the virtual lanes t, t + blockDim.x, ... below 128 (two at 64 threads, none above 127 at 256), and
 // issues all its loads of a round before it adds (one L2 round trip for up to 8 entries per lane);
-// thread 0 divides (FP64, once per block).  DF: the partials are double-FP32 pairs (hi, lo) in the 8
+// thread 0 divides (once per block).  DF: the partials are double-FP32 pairs (hi, lo) in the 8
 // bytes of each entry, added with TwoSum on the FP32 pipes (the FP32 and double-FP32 solves; GB300's
 // FP64 pipe is 1/64 of the FP32 rate), else FP64 values added in FP64.
 // x: the numerator (denominator) value, loaded by the caller together with its other loads, so
@@ -767,10 +767,12 @@ struct PartialsRatio {
   int stop;
 };
 
-// (hi, lo) pair combined over the 32 lanes of a warp in a fixed tree; valid in lane 0
+// (hi, lo) pairs of N lanes (a power of two; the rest hold zeros or are ignored) combined in a fixed tree; valid in
+// lane 0.  A tree over 32 lanes with zeros beyond N gives the same bits: each level takes some 75 clocks.
+template <int N = 32>
 __device__ __forceinline__ float2 warp_tree_df(float2 v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = N / 2; o > 0; o >>= 1) {
     const float oh = __shfl_down_sync(0xffffffffu, v.x, o), ol = __shfl_down_sync(0xffffffffu, v.y, o);
     float s = v.x, c = v.y;
     df_add(s, c, oh, ol);
@@ -779,9 +781,10 @@ __device__ __forceinline__ float2 warp_tree_df(float2 v) {
   return v;
 }
 
+template <int N = 32>
 __device__ __forceinline__ double warp_tree64(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  for (int o = N / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
 
@@ -812,7 +815,7 @@ __device__ __forceinline__ PartialsRatio partials_ratio64(const double* partials
     return r;
   }
   if (t < 32) {
-    const double u = warp_tree64(t < kSumLanes / 32 ? gsum[t] : 0.0);
+    const double u = warp_tree64<kSumLanes / 32>(t < kSumLanes / 32 ? gsum[t] : 0.0);
     if (t == 0) {
       const double q = SUM_OVER_X ? u / x : x / u;
       res.sum = u;
@@ -859,7 +862,7 @@ __device__ __forceinline__ PartialsRatio partials_ratio_df(const double* partial
     return r;
   }
   if (t < 32) {
-    const float2 u = warp_tree_df(t < kSumLanes / 32 ? gsum[t] : make_float2(0.f, 0.f));
+    const float2 u = warp_tree_df<kSumLanes / 32>(t < kSumLanes / 32 ? gsum[t] : make_float2(0.f, 0.f));
     if (t == 0) {
       const DfPair q = SUM_OVER_X ? df_div_pair(u.x, u.y, x.x, x.y) : df_div_pair(x.x, x.y, u.x, u.y);
       res.sum_df = u;
@@ -876,10 +879,12 @@ __device__ __forceinline__ PartialsRatio partials_ratio_df(const double* partial
   return res;
 }
 
+constexpr int kMaxWarps = 8;  // blocks of at most 256 threads
+
 // Sum over the block of per-thread FP32 values as a double-FP32 pair: in FP32 within each warp (a fixed
 // xor tree, as block_sum_mixed), across the warps with TwoSum in a fixed tree; valid in thread 0.
 __device__ __forceinline__ float2 block_sum_f_df(float v) {
-  __shared__ float2 red_fd[32];
+  __shared__ float2 red_fd[kMaxWarps];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -887,20 +892,20 @@ __device__ __forceinline__ float2 block_sum_f_df(float v) {
   if (l == 0) red_fd[w] = make_float2(v, 0.f);
   __syncthreads();
   float2 u = make_float2(0.f, 0.f);
-  if (w == 0) u = warp_tree_df(l < nw ? red_fd[l] : make_float2(0.f, 0.f));
+  if (w == 0) u = warp_tree_df<kMaxWarps>(l < nw ? red_fd[l] : make_float2(0.f, 0.f));
   return u;
 }
 
 // The same for per-thread double-FP32 values (s, c): TwoSum shuffle trees within and across the warps.
 __device__ __forceinline__ float2 block_sum_df_df(float s, float c) {
-  __shared__ float2 red_dd[32];
+  __shared__ float2 red_dd[kMaxWarps];
   float2 v = warp_tree_df(df_norm(s, c));
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
   __syncthreads();
   if (l == 0) red_dd[w] = v;
   __syncthreads();
   v = make_float2(0.f, 0.f);
-  if (w == 0) v = warp_tree_df(l < nw ? red_dd[l] : make_float2(0.f, 0.f));
+  if (w == 0) v = warp_tree_df<kMaxWarps>(l < nw ? red_dd[l] : make_float2(0.f, 0.f));
   return v;
 }
 

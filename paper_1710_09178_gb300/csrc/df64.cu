@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(256, 4) df_r_update_kernel(Geom g, const __gri
   const float2 rr_df = sd->rr_df;
   const int vh = g.vh;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nb = (vh + 255) / 256;  // then the scalar block, then a block per shift for its recurrence
+  const int nb = (vh + blockDim.x - 1) / blockDim.x;  // then the scalar block, then one per shift for its recurrence
   const bool scalar_block = (int)blockIdx.x == nb;
   if ((int)blockIdx.x > nb) {
     if (!__syncthreads_or(skip)) window_scalars_shift<false>(sd, blockIdx.x - nb - 1);

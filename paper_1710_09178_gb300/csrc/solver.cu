@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(256, 4) r_update_kernel(Geom g, const __grid_c
   const double rr = sd->rr;
   const float2 rr_df = sd->rr_df;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nb = (g.vh + 255) / 256;  // then the scalar block, then a block per shift for its recurrence
+  const int nb = (g.vh + blockDim.x - 1) / blockDim.x;  // then the scalar block, then one per shift for its recurrence
   const bool scalar_block = (int)blockIdx.x == nb;
   if ((int)blockIdx.x > nb) {
     if (!__syncthreads_or(skip)) window_scalars_shift<false>(sd, blockIdx.x - nb - 1);
