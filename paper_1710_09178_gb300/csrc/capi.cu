@@ -142,6 +142,12 @@ int lqcd_share_gauge(lqcd_ctx* ctx, const lqcd_ctx* src) {
 
 int lqcd_set_gauge(lqcd_ctx* ctx, const double* U_dev) {
   if (!ctx) return LQCD_ERR_ARG;
+  return lqcd::set_gauge(ctx, U_dev, true);
+}
+
+}  // extern "C"
+
+int lqcd::set_gauge(lqcd_ctx* ctx, const double* U_dev, bool all) {
   if (!U_dev) return fail(ctx, LQCD_ERR_ARG, "lqcd_set_gauge: null gauge pointer");
   if (!ctx->gauge.owned) return fail(ctx, LQCD_ERR_STATE, "lqcd_set_gauge: this context borrows its gauge field");
   Geom g = make_geom(ctx);
@@ -182,12 +188,19 @@ int lqcd_set_gauge(lqcd_ctx* ctx, const double* U_dev) {
     gc.u16 = at + off[5];
     if (fix) gc.ufix = reinterpret_cast<int4*>(at + off[6]);
   }
-  e = launch_pack_gauge(g, reinterpret_cast<const double2*>(U_dev), gc, ctx->stream);
+  GaugeCopies dst = gc;
+  if (!all) {
+    dst.u8 = nullptr;
+    dst.u16 = nullptr;
+  }
+  e = launch_pack_gauge(g, reinterpret_cast<const double2*>(U_dev), dst, ctx->stream);
   ctx->launches += 1;
   if (e != cudaSuccess) return cuda_check(ctx, e, "pack_gauge");
   gc.loaded = true;
   return LQCD_OK;
 }
+
+extern "C" {
 
 size_t lqcd_vector_bytes(const lqcd_ctx* ctx, int prec) {
   if (!ctx) return 0;

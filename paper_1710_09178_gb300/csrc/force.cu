@@ -207,7 +207,6 @@ extern "C" int fermion_force(lqcd_ctx* ctx, const double* shifts, const double* 
   if (rc != LQCD_OK) return rc;
   Geom g = make_geom(ctx);
   cudaStream_t st = workspace_stream(ctx);
-  double2* const* xs = workspace_solutions(ctx);
   const bool dbl = prec == LQCD_FP64;
   ForceWorkspace* fw = static_cast<ForceWorkspace*>(ctx->force_ws);
   cudaError_t e;
@@ -231,6 +230,11 @@ extern "C" int fermion_force(lqcd_ctx* ctx, const double* shifts, const double* 
   }
   const int n3 = 3 * g.vh;
   int nl = 0;
+  // the FP32 adjoint takes X_k rounded to FP32: the hi parts where the solve left (hi, lo) pairs
+  void* const* hi = dbl ? nullptr : workspace_pairs(ctx);
+  double2* const* xs = nullptr;
+  auto need_xs = [&]() -> int { return xs ? LQCD_OK : workspace_solutions(ctx, &xs); };
+  if (!hi && (rc = need_xs()) != LQCD_OK) return rc;
   ForceArgs fa;
   memset(&fa, 0, sizeof(fa));
   fa.n = n;
@@ -244,14 +248,16 @@ extern "C" int fermion_force(lqcd_ctx* ctx, const double* shifts, const double* 
       d.prec = LQCD_FP64;
       fa.x[k] = xs[k];
     } else {
-      narrow_kernel<<<(n3 + 255) / 256, 256, 0, st>>>(n3, xs[k], static_cast<float2*>(fw->x32[k]));
-      nl += 1;
-      d.in = fw->x32[k];
+      if (!hi) {
+        narrow_kernel<<<(n3 + 255) / 256, 256, 0, st>>>(n3, xs[k], static_cast<float2*>(fw->x32[k]));
+        nl += 1;
+      }
+      d.in = hi ? hi[k] : fw->x32[k];
       d.prec = LQCD_FP32;
       d.tps = ctx->dslash_tps;
       d.bs = ctx->dslash_bs;
       d.order = ctx->dslash_order;
-      fa.x[k] = fw->x32[k];
+      fa.x[k] = d.in;
     }
     if ((e = launch_dslash(g, ctx->gauge, d, st, &nl)) != cudaSuccess) return cuda_check(ctx, e, "fermion_force");
     fa.y[k] = fw->y[k];
@@ -267,6 +273,7 @@ extern "C" int fermion_force(lqcd_ctx* ctx, const double* shifts, const double* 
     nl += 1;
   }
   if (action_host) {
+    if ((rc = need_xs()) != LQCD_OK) return rc;
     ActionArgs aa;
     memset(&aa, 0, sizeof(aa));
     aa.phi = reinterpret_cast<const double2*>(phi_dev);

@@ -144,6 +144,9 @@ Geom make_geom(const lqcd_ctx* ctx);
 int fail(lqcd_ctx* ctx, int code, const std::string& msg);
 int cuda_check(lqcd_ctx* ctx, cudaError_t e, const char* what);
 
+// capi.cu: lqcd_set_gauge; with all false, without the 8-real and 16-bit copies (which keep an earlier field)
+int set_gauge(lqcd_ctx* ctx, const double* U_dev, bool all);
+
 // pack.cu
 cudaError_t launch_pack_gauge(const Geom& g, const double2* U, GaugeCopies& gc, cudaStream_t st);
 cudaError_t launch_pack_vector(const Geom& g, void* dst, int prec, const double2* src, cudaStream_t st);
@@ -281,8 +284,10 @@ int run_mshift_multi(lqcd_ctx* ctx, int S, const double* shifts, const double* r
                      const double* const* b_devs, double* const* const* x_devs, double* const* y_devs, double tol,
                      int maxiter, int prec, lqcd_solve_stats* stats);
 void free_workspace(lqcd_ctx* ctx);
-// FP64 internal solutions x_k of the last mshift_cg call on this context, and its stream
-double2* const* workspace_solutions(lqcd_ctx* ctx);
+// After an mshift_cg call on this context, on its stream: its solutions as FP64 vectors (converted where the solve left
+// them as pairs), or as the (hi, lo) pairs it left (null: none; workspace_solutions ends their time)
+int workspace_solutions(lqcd_ctx* ctx, double2* const** xs);
+void* const* workspace_pairs(lqcd_ctx* ctx);
 cudaStream_t workspace_stream(lqcd_ctx* ctx);
 
 // force.cu, trajectory.cu

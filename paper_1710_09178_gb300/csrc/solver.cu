@@ -558,9 +558,19 @@ __global__ void axpy64_kernel(int n3, double2* __restrict__ x, const double2* __
   x[i] = make_double2(a.x + b.x, a.y + b.y);
 }
 
-// canonical outputs: x_k unpacked, y = c0 b + sum_k c_k x_k (FP64)
+// An FP32 number as FP64 by integer operations: the conversion instruction runs on the FP64 pipe, 2 lanes per clock and
+// SM.  Exact; zeros, denormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if (e == 0u || e == 255u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+// canonical outputs: x_k unpacked, y = c0 b + sum_k c_k x_k (FP64).  One thread per complex component, in the order of
+// the outputs.  PAIRS: x_k as (hi, lo) FP32 pairs (x = hi + lo), else FP64.  32^3x8 with 16 shifts: 108 us for 205 MB read
+// and written (with the pairs' conversion in a kernel of its own before: 155 us and 400 MB); of that 41 us of FP64 pipe.
 struct OutArgs {
-  const double2* xk[kMaxShifts];
+  const void* xk[kMaxShifts];
   double2* xout[kMaxShifts];
   double c[kMaxShifts];
   double c0;
@@ -569,21 +579,40 @@ struct OutArgs {
   int n;
 };
 
-__global__ void outputs_kernel(Geom g, OutArgs a) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.vh) return;
-  int vh = g.vh;
-  for (int c = 0; c < 3; ++c) {
-    double2 b = a.b64[c * vh + i];
-    double yr = a.c0 * b.x, yi = a.c0 * b.y;
-    for (int k = 0; k < a.n; ++k) {
-      double2 x = a.xk[k][c * vh + i];
-      if (a.xout[k]) a.xout[k][3 * (size_t)i + c] = x;
-      yr += a.c[k] * x.x;
-      yi += a.c[k] * x.y;
+template <bool PAIRS>
+__global__ void __launch_bounds__(256) outputs_kernel(int vh, const __grid_constant__ OutArgs a) {
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n3 = 3 * vh;
+  if (e >= (unsigned)n3) return;
+  const unsigned i = e / 3u, c = e - 3u * i, o = c * (unsigned)vh + i;
+  const double2 b = a.b64[o];
+  double yr = a.c0 * b.x, yi = a.c0 * b.y;
+  constexpr int kBatch = 4;  // shifts whose loads are in flight together (the stores could alias them, says the type)
+  for (int k0 = 0; k0 < a.n; k0 += kBatch) {
+    float2 h[kBatch], l[kBatch];
+    double2 x[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      if (k0 + q >= a.n) break;
+      if constexpr (PAIRS) {
+        const float2* v = static_cast<const float2*>(a.xk[k0 + q]);
+        h[q] = __ldg(v + o);
+        l[q] = __ldg(v + o + n3);
+      } else {
+        x[q] = __ldg(static_cast<const double2*>(a.xk[k0 + q]) + o);
+      }
     }
-    if (a.y) a.y[3 * (size_t)i + c] = make_double2(yr, yi);
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int k = k0 + q;
+      if (k >= a.n) break;
+      if constexpr (PAIRS) x[q] = make_double2(widen(h[q].x) + widen(l[q].x), widen(h[q].y) + widen(l[q].y));
+      if (a.xout[k]) a.xout[k][e] = x[q];
+      yr = fma(a.c[k], x[q].x, yr);
+      yi = fma(a.c[k], x[q].y, yi);
+    }
   }
+  if (a.y) a.y[e] = make_double2(yr, yi);
 }
 
 __global__ void zero_kernel(int n3, double2* __restrict__ x) {
@@ -614,6 +643,7 @@ struct Workspace {
   double2* xk[kMaxShifts] = {};
   void* xdf[kMaxShifts] = {};  // the solutions as (hi, lo) FP32 pairs during the solve (xdfmode)
   bool xdfmode = false;        // every mode but LQCD_FP64 (with double-FP32 residuals)
+  int pairs = 0;               // the last solve left this many solutions as pairs only (xk is not current)
   double2 *b64 = nullptr, *r64 = nullptr, *tmp64 = nullptr, *e64 = nullptr, *rb64 = nullptr;
   // double-FP32 residuals (mixed modes): x, D_oe x and b as (hi, lo) pairs
   bool df = false;
@@ -656,7 +686,6 @@ static size_t vec_bytes(long long vh, int prec) {
   return 0;
 }
 
-double2* const* workspace_solutions(lqcd_ctx* ctx) { return ctx->ws ? ctx->ws->xk : nullptr; }
 cudaStream_t workspace_stream(lqcd_ctx* ctx) { return ctx->ws ? ctx->ws->st : nullptr; }
 
 static void destroy_workspace(Workspace* w) {
@@ -1888,10 +1917,8 @@ int run_mshift_multi(lqcd_ctx* ctx, int S, const double* shifts, const double* r
         for (int k = 0; k < n; ++k)
           if (!(tres[s][k] <= tol)) status = LQCD_ERR_NOT_CONVERGED;
     }
-    if (y->xdfmode && bb != 0.0) {
-      LQ_CUDA(launch_df_to_fp64_many(g, y->xdf, y->xk, n, w->st));
-      ctx->launches += 1;
-    }
+    const bool pairs = y->xdfmode && bb != 0.0;
+    y->pairs = pairs ? n : 0;
     if (bb == 0.0) {
       for (int k = 0; k < n; ++k) {
         zero_kernel<<<(3 * g.vh + 255) / 256, 256, 0, w->st>>>(3 * g.vh, y->xk[k]);
@@ -1901,17 +1928,23 @@ int run_mshift_multi(lqcd_ctx* ctx, int S, const double* shifts, const double* r
     // outputs in the canonical layout
     OutArgs oa;
     memset(&oa, 0, sizeof(oa));
+    bool any = false;
     for (int k = 0; k < n; ++k) {
-      oa.xk[k] = y->xk[k];
+      oa.xk[k] = pairs ? y->xdf[k] : y->xk[k];
       oa.xout[k] = x_devs && x_devs[s] ? reinterpret_cast<double2*>(x_devs[s][k]) : nullptr;
+      any = any || oa.xout[k];
       oa.c[k] = residues ? residues[k] : 0.0;
     }
     oa.c0 = c0;
     oa.b64 = y->b64;
     oa.y = y_devs ? reinterpret_cast<double2*>(y_devs[s]) : nullptr;
     oa.n = n;
-    outputs_kernel<<<(g.vh + 255) / 256, 256, 0, w->st>>>(g, oa);
-    ctx->launches += 1;
+    if (any || oa.y) {
+      const unsigned nb3 = (unsigned)((3 * g.vh + 255) / 256);
+      if (pairs) outputs_kernel<true><<<nb3, 256, 0, w->st>>>(g.vh, oa);
+      else outputs_kernel<false><<<nb3, 256, 0, w->st>>>(g.vh, oa);
+      ctx->launches += 1;
+    }
     LQ_CUDA(cudaGetLastError());
     core[s].status = status;
     if (status_all == LQCD_OK && status != LQCD_OK) status_all = status;
@@ -1945,6 +1978,19 @@ int run_mshift_multi(lqcd_ctx* ctx, int S, const double* shifts, const double* r
   if (status_all != LQCD_OK) return fail(ctx, status_all, "shifted CG failed");
   return LQCD_OK;
 }
+
+int workspace_solutions(lqcd_ctx* ctx, double2* const** xs) {
+  Workspace* w = ctx->ws;
+  if (w->pairs) {
+    LQ_CUDA(launch_df_to_fp64_many(make_geom(ctx), w->xdf, w->xk, w->pairs, w->st));
+    ctx->launches += 1;
+    w->pairs = 0;
+  }
+  *xs = w->xk;
+  return LQCD_OK;
+}
+
+void* const* workspace_pairs(lqcd_ctx* ctx) { return ctx->ws && ctx->ws->pairs ? ctx->ws->xdf : nullptr; }
 
 int run_mshift(lqcd_ctx* ctx, const double* shifts, const double* residues, int n, double c0, const double* b_dev,
                double* const* x_dev, double* y_dev, double tol, int maxiter, int prec, lqcd_solve_stats* stats) {

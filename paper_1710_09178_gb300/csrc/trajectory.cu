@@ -525,11 +525,26 @@ extern "C" int rhmc_trajectory(lqcd_ctx* ctx, const lqcd_rhmc_params* prm, doubl
     TJ_CUDA(cudaGetLastError());
     return LQCD_OK;
   };
+  struct Links {  // every copy of the context's field is that of tw->U again on each way out
+    lqcd_ctx* ctx;
+    const double2* U;
+    bool stale;
+    int finish() {
+      if (!stale) return LQCD_OK;
+      stale = false;
+      return set_gauge(ctx, reinterpret_cast<const double*>(U), true);
+    }
+    ~Links() { finish(); }
+  } links{ctx, tw->U, false};
   auto drift = [&](double h) -> int {
     link_update_kernel<<<nbl, 128, 0, st>>>(4 * V, tw->U, tw->P, h);
     nl += 1;
     TJ_CUDA(cudaGetLastError());
-    return lqcd_set_gauge(ctx, reinterpret_cast<const double*>(tw->U));
+    // the compact copies that the trajectory's solves do not read follow at its end
+    const bool all = prm->prec == LQCD_FP32_R8 || prm->prec == LQCD_FP32_L16 || prm->prec_action == LQCD_FP32_R8 ||
+                     prm->prec_action == LQCD_FP32_L16;
+    links.stale = !all;
+    return set_gauge(ctx, reinterpret_cast<const double*>(tw->U), all);
   };
   if ((rc = hamiltonian(&res->kinetic0, &res->gauge0, &res->fermion0)) != LQCD_OK) return rc;
   // Omelyan 2MN
@@ -551,9 +566,11 @@ extern "C" int rhmc_trajectory(lqcd_ctx* ctx, const lqcd_rhmc_params* prm, doubl
   res->accepted = (uniform < exp(-res->dH)) ? 1 : 0;
   if (!std::isfinite(res->dH)) res->accepted = 0;
   if (res->accepted) {
+    if ((rc = links.finish()) != LQCD_OK) return rc;
     TJ_CUDA(cudaMemcpyAsync(U_dev, tw->U, sizeof(double2) * 9 * 4 * V, cudaMemcpyDeviceToDevice, st));
-  } else if ((rc = lqcd_set_gauge(ctx, U_dev)) != LQCD_OK) {
-    return rc;
+  } else {
+    links.stale = false;
+    if ((rc = lqcd_set_gauge(ctx, U_dev)) != LQCD_OK) return rc;
   }
   if (prm->mom_out) TJ_CUDA(cudaMemcpyAsync(prm->mom_out, tw->P, sizeof(double) * ncomp, cudaMemcpyDeviceToDevice, st));
   if (prm->links_out)
