@@ -95,6 +95,13 @@ __device__ __forceinline__ float2 df_a(const DfArgs& k) {
   return k.a_split ? make_float2(k.a_hi, k.a_lo) : (k.a_devdf ? *k.a_devdf : split64(k.a_dev ? *k.a_dev : k.a));
 }
 
+// (yh + yl) + a (xh + xl) as a normalised pair
+__device__ __forceinline__ float2 df_axpy(float yh, float yl, float2 a, float xh, float xl) {
+  float s = yh, c = yl;
+  df_mac(s, c, a.x, a.y, xh, xl);
+  return df_norm(s, c);
+}
+
 // What the epilogues read at the output site beside the hops' sum, for one colour.
 struct DfOwn {
   float2 xh, xl, bh, bl;
@@ -173,15 +180,19 @@ __device__ __forceinline__ void df_reduce(const DfArgs& k, float ds, float dc) {
 // The block holds NS = blockDim.x / TPS sites; thread t takes directions t / NS ND .. of site t % NS, ND = 4 / TPS.
 // The four sums meet in shared memory (which with TPS = 1 also keeps them out of the registers that the
 // next links are loaded into), and thread sub finishes colours sub, sub + TPS, ..
-template <int EPI, int TPS>
-__global__ void __launch_bounds__(kDfThreads, 4) df_dslash_kernel(Geom g, const __grid_constant__ PerSys<DfArgs> pk) {
+// UPD: the p update folded in (small lattices, one system): EPI 0 takes r + beta in at every neighbour, beta summed from the
+// r update's partials as the p update kernel does, and runs the beta step in the last block; EPI 1 takes r + beta x at its
+// own site and stores it in x.  The same operations, the same bits.
+template <int EPI, int TPS, bool UPD>
+__global__ void __launch_bounds__(kDfThreads, UPD ? 2 : 4) df_dslash_kernel(Geom g, const __grid_constant__ PerSys<DfArgs> pk) {
   constexpr int NS = kDfThreads / TPS, ND = 4 / TPS;
   __shared__ float4 part[4][3][NS];
   const DfArgs& k = pk.s[blockIdx.y];
   const int vh = g.vh;
   const int sub = threadIdx.x / NS, ls = threadIdx.x % NS;
   const int i = blockIdx.x * NS + ls;
-  const bool valid = i < vh;
+  const bool scalar_block = UPD && EPI == 0 && blockIdx.x == gridDim.x - 1;
+  const bool valid = !scalar_block && i < vh;
   const int p = k.out_parity;
   const uint64_t pol_hi = policy_evict_last();   // the solver's FP32 links: keep them in L2
   const uint64_t pol_lo = policy_evict_first();  // rounding errors, read only by the checks
@@ -198,7 +209,34 @@ __global__ void __launch_bounds__(kDfThreads, 4) df_dslash_kernel(Geom g, const 
   }
   pdl_wait();
   pdl_trigger();
-  if ((k.done && *k.done) || (k.halt && *k.halt)) return;  // uniform
+  float2 be = make_float2(0.f, 0.f);
+  Vec3<float> rh[2], rl[2], ph[2], pl[2];  // UPD: r and p at the first direction's neighbours
+  auto load_rp = [&](int q, int j) {
+    rh[q] = load_vec(k.upd_r, j, vh);
+    rl[q] = load_vec(k.upd_r + 3 * (size_t)vh, j, vh);
+    ph[q] = load_vec(k.in_hi, j, vh);
+    pl[q] = load_vec(k.in_lo, j, vh);
+  };
+  if constexpr (UPD && EPI == 0) {
+    SolverDev* sd = k.sd;
+    // the scalar block may set done meanwhile: partials_ratio settles the block on one reading
+    const bool skip = (*reinterpret_cast<const volatile int*>(&sd->done) | (k.halt ? *k.halt : 0)) != 0;
+    const float2 rr_b_df = sd->rr_b_df;
+    if (valid) {
+      load_rp(0, neighbour_half(g, neighbour_fwd(g, s, sub * ND)));
+      load_rp(1, neighbour_half(g, neighbour_bwd(g, s, sub * ND)));
+    }
+    const PartialsRatio pb = partials_ratio_df<true>(k.rr_partials, k.n_rr, rr_b_df, skip, scalar_block);
+    if (pb.stop) return;  // the same in every thread of the block
+    if (scalar_block) {
+      solver_beta_step(sd, pb);
+      return;
+    }
+    be = pb.ratio_df;
+  } else {
+    if ((k.done && *k.done) || (k.halt && *k.halt)) return;  // uniform
+    if constexpr (UPD) be = k.sd->beta_df;
+  }
 
   constexpr int NC = (3 + TPS - 1) / TPS;  // colours finished by thread sub: sub, sub + TPS, ..
   DfOwn own[NC];
@@ -207,7 +245,18 @@ __global__ void __launch_bounds__(kDfThreads, 4) df_dslash_kernel(Geom g, const 
     if (EPI != 0) asp = df_a(k);
 #pragma unroll
     for (int q = 0; q < NC; ++q)
-      if (valid && sub + q * TPS < 3) own[q] = df_own<EPI>(k, (size_t)(sub + q * TPS) * vh + i);
+      if (valid && sub + q * TPS < 3) {
+        const size_t o = (size_t)(sub + q * TPS) * vh + i;
+        own[q] = df_own<EPI>(k, o);
+        if constexpr (UPD && EPI == 1) {
+          const float2 re = df_axpy(k.upd_r[o].x, k.upd_r[o + 3 * (size_t)vh].x, be, own[q].xh.x, own[q].xl.x),
+                       im = df_axpy(k.upd_r[o].y, k.upd_r[o + 3 * (size_t)vh].y, be, own[q].xh.y, own[q].xl.y);
+          own[q].xh = make_float2(re.x, im.x);
+          own[q].xl = make_float2(re.y, im.y);
+          const_cast<float2*>(k.x_hi)[o] = own[q].xh;
+          const_cast<float2*>(k.x_lo)[o] = own[q].xl;
+        }
+      }
   };
   if (TPS > 1) load_own();
   if (valid) {
@@ -224,7 +273,20 @@ __global__ void __launch_bounds__(kDfThreads, 4) df_dslash_kernel(Geom g, const 
           Uh = load_link32(k.links_hi, lp, mu, li, vh, pol_hi);
           Ul = load_link32(k.links_lo, lp, mu, li, vh, pol_lo);
         }
-        const Vec3<float> vh3 = ldg_vec(k.in_hi, j, vh), vl3 = ldg_vec(k.in_lo, j, vh);
+        Vec3<float> vh3, vl3;
+        if constexpr (UPD && EPI == 0) {
+          if (d > 0) load_rp(h, j);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float2 re = df_axpy(rh[h].c[c].re, rl[h].c[c].re, be, ph[h].c[c].re, pl[h].c[c].re),
+                         im = df_axpy(rh[h].c[c].im, rl[h].c[c].im, be, ph[h].c[c].im, pl[h].c[c].im);
+            vh3.c[c] = cmake(re.x, im.x);
+            vl3.c[c] = cmake(re.y, im.y);
+          }
+        } else {
+          vh3 = ldg_vec(k.in_hi, j, vh);
+          vl3 = ldg_vec(k.in_lo, j, vh);
+        }
         df_hop(sr, cr, si, ci, Uh, Ul, vh3, vl3, fwd);
       }
 #pragma unroll
@@ -275,10 +337,19 @@ int df_dslash_grid_blocks(const Geom& g) {
 template <int TPS>
 static cudaError_t launch_df_tps(const Geom& g, const PerSys<DfArgs>& a, int S, int epi, cudaStream_t st, bool pdl) {
   const dim3 grid((unsigned)df_dslash_grid_blocks(g), (unsigned)S), block(kDfThreads);
-  if (epi == 2) return launch_k(pdl, df_dslash_kernel<2, TPS>, grid, block, st, g, a);
-  if (epi == 1) return launch_k(pdl, df_dslash_kernel<1, TPS>, grid, block, st, g, a);
-  return launch_k(pdl, df_dslash_kernel<0, TPS>, grid, block, st, g, a);
+  if constexpr (TPS > 1) {
+    if (a.s[0].upd_r) {
+      if (S != 1 || epi == 2) return cudaErrorInvalidValue;
+      if (epi == 1) return launch_k(pdl, df_dslash_kernel<1, TPS, true>, grid, block, st, g, a);
+      return launch_k(pdl, df_dslash_kernel<0, TPS, true>, dim3(grid.x + 1), block, st, g, a);
+    }
+  }
+  if (epi == 2) return launch_k(pdl, df_dslash_kernel<2, TPS, false>, grid, block, st, g, a);
+  if (epi == 1) return launch_k(pdl, df_dslash_kernel<1, TPS, false>, grid, block, st, g, a);
+  return launch_k(pdl, df_dslash_kernel<0, TPS, false>, grid, block, st, g, a);
 }
+
+bool fold_df_p_update(const Geom& g) { return df_tps(g) > 1; }
 
 cudaError_t launch_df_dslash_multi(const Geom& g, const PerSys<DfArgs>& a, int S, int epi, cudaStream_t st, bool pdl) {
   switch (df_tps(g)) {

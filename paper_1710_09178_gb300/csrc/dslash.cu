@@ -18,6 +18,7 @@
 #include "common.cuh"
 #include "fix64.cuh"
 #include "internal.h"
+#include "solver_dev.cuh"
 
 namespace lqcd {
 
@@ -42,6 +43,10 @@ struct KArgs {
   const void* links;
   const double2* links64;  // FP64 only: the copy behind the fixed-point one
   int order;  // block-to-site order (site_block)
+  const void* upd_r;  // the p update folded in (DslashArgs)
+  SolverDev* sd;
+  const double* rr_partials;
+  int n_rr;
 };
 
 // A link as loaded from memory (the compact forms stay compact while their loads are in flight)
@@ -126,7 +131,8 @@ __device__ __forceinline__ void dslash_reduce(const KArgs& k, T dsite) {
 // Output stage shared by the Dslash kernels: d = (D in)(x) of site i, written as the plain
 // output, the A-apply a * aux - d with Re<aux, out>, or the residual bvec - (a * aux - d) with
 // |out|^2; the sums are reduced over the grid by the last block (every thread of the block calls).
-template <typename T, typename V2, int TPS, int EPI>
+// UPD: the A-apply may have the p update folded in (k.upd_r).
+template <typename T, typename V2, int TPS, int EPI, bool UPD = false>
 __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d, int i, int sub, bool valid,
                                                 int vh) {
   V2* out = static_cast<V2*>(k.out);
@@ -148,6 +154,15 @@ __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d
         out[o] = w;
       } else {
         V2 ps = static_cast<const V2*>(k.aux)[o];
+        if constexpr (UPD && EPI == (int)Epi::AApply) {
+          if (k.upd_r) {  // uniform: p = r + beta p, as the p update kernel forms it
+            const T beta = (T)k.sd->beta_f;
+            const V2 r = static_cast<const V2*>(k.upd_r)[o];
+            ps.x = fma(beta, ps.x, r.x);
+            ps.y = fma(beta, ps.y, r.y);
+            static_cast<V2*>(const_cast<void*>(k.aux))[o] = ps;
+          }
+        }
         T qre = aval * ps.x - d.c[c].re;
         T qim = aval * ps.y - d.c[c].im;
         if constexpr (EPI == (int)Epi::AApply) {
@@ -247,9 +262,14 @@ struct SiteHopsAhead {
   }
 
   __device__ __forceinline__ Vec3<float> apply(const void*, const float2* in, int, int, int, int vh, uint64_t) {
-    Vec3<float> v[8], accf = vzero<float>(), accb = vzero<float>();
+    Vec3<float> v[8];
 #pragma unroll
     for (int h = 0; h < 8; ++h) v[h] = ldg_vec(in, nb[h], vh);
+    return apply_to(v);
+  }
+
+  __device__ __forceinline__ Vec3<float> apply_to(const Vec3<float> (&v)[8]) const {
+    Vec3<float> accf = vzero<float>(), accb = vzero<float>();
 #pragma unroll
     for (int h = 0; h < 8; ++h) {
       const Mat3<float> M = decode<LF>(W[h], sg[h]);
@@ -312,7 +332,60 @@ __global__ void __launch_bounds__(128, AHEAD ? 1 : 7) dslash_kernel(Geom g, KArg
     d.c[c] = cmake(re, im);
   }
 
-  dslash_epilogue<T, V2, TPS, EPI>(k, d, i, sub, valid, vh);
+  dslash_epilogue<T, V2, TPS, EPI, AHEAD>(k, d, i, sub, valid, vh);
+}
+
+// The plain hop with the p update folded in (small lattices, one system): in is the p before it.  While the links and
+// vectors are on their way, every block sums the r update's partials as the p update kernel does (the same beta, so the
+// same bits); the last block runs the beta step.  A launch and a round trip less per iteration: p_update takes 1.4 us and
+// a launch gap of 0.9, the sum here about 0.8.
+template <int LF>
+__global__ void __launch_bounds__(128, 1) dslash_pupdate_kernel(Geom g, KArgs k) {
+  __shared__ __align__(8) float2 rs[8][3][128];  // each thread's neighbours of r (registers hold p and the links)
+  const int vh = g.vh, t = threadIdx.x, p = k.out_parity;
+  const bool scalar_block = blockIdx.x == gridDim.x - 1;
+  const int i = blockIdx.x * 128 + t;
+  const bool valid = !scalar_block && i < vh;
+  const float2* in = static_cast<const float2*>(k.in);
+  const float2* r = static_cast<const float2*>(k.upd_r);
+  SiteHopsAhead<LF> hops;
+  if (valid) hops.start(g, k.links, p, i, 0, policy_evict_last());
+  pdl_wait();
+  pdl_trigger();
+  SolverDev* sd = k.sd;
+  const bool skip = *reinterpret_cast<const volatile int*>(&sd->done) != 0;
+  const float2 rr_b_df = sd->rr_b_df;
+  Vec3<float> v[8];
+  if (valid) {
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(&rs[h][c][t])),
+                     "l"(r + (size_t)c * vh + hops.nb[h])
+                     : "memory");
+      v[h] = load_vec(in, hops.nb[h], vh);
+    }
+  }
+  const PartialsRatio pb = partials_ratio_df<true>(k.rr_partials, k.n_rr, rr_b_df, skip, scalar_block);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (pb.stop) return;  // the same in every thread of the block
+  if (scalar_block) {
+    solver_beta_step(sd, pb);
+    return;
+  }
+  if (!valid) return;
+  const float beta = pb.ratio_f;
+#pragma unroll
+  for (int h = 0; h < 8; ++h) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2 w = rs[h][c][t];
+      v[h].c[c].re = fma(beta, v[h].c[c].re, w.x);
+      v[h].c[c].im = fma(beta, v[h].c[c].im, w.y);
+    }
+  }
+  store_vec(static_cast<float2*>(k.out), i, vh, hops.apply_to(v));
 }
 
 // FP64: the products in block fixed point (fix64.cuh), one direction per thread.  Blocks take groups of
@@ -576,6 +649,7 @@ static cudaError_t launch_tps(const Geom& g, const KArgs& k, Epi epi, cudaStream
   // 20^3x8 (250) 3.07 and 3.20, 24^3x6 (324) 3.37 and 4.72.
   if constexpr (TPS == 1) {
     if (nb <= kSMs) {
+      if (epi == Epi::Plain && k.upd_r) return launch_k(pdl, dslash_pupdate_kernel<LF>, dim3(nb + 1), dim3(128), st, g, k);
       switch (epi) {
         case Epi::Plain: return launch_k(pdl, dslash_kernel<LF, 1, 0, true>, dim3(nb), dim3(bs), st, g, k);
         case Epi::AApply: return launch_k(pdl, dslash_kernel<LF, 1, 1, true>, dim3(nb), dim3(bs), st, g, k);
@@ -614,6 +688,10 @@ static cudaError_t launch_fp64(const Geom& g, const KArgs& k, Epi epi, cudaStrea
 
 static int default_tps(int) { return 1; }  // fastest on GB300 at 16^3x8 and 32^3x8 (sweep over 1, 2, 4, 8)
 
+bool fold_p_update(const Geom& g, int tps, int bs, int order) {
+  return (tps <= 0 ? default_tps(LQCD_FP32) : tps) == 1 && (bs <= 0 || bs == 128) && order == 0 && (g.vh + 127) / 128 <= kSMs;
+}
+
 // blocks of one Dslash launch (= partials it writes)
 int dslash_grid_blocks(const Geom& g, int prec, int tps, int bs) {
   if (prec == LQCD_FP64) return fp64_blocks(g);
@@ -642,6 +720,11 @@ cudaError_t launch_dslash(const Geom& g, const GaugeCopies& gc, const DslashArgs
   const int bs = a.bs > 0 ? a.bs : 128;
   if (bs != 64 && bs != 128) return cudaErrorInvalidValue;
   k.order = (a.prec == LQCD_FP64) ? 0 : a.order;
+  k.upd_r = a.upd_r;
+  k.sd = a.sd;
+  k.rr_partials = a.rr_partials;
+  k.n_rr = a.n_rr;
+  if (k.upd_r && (a.prec == LQCD_FP64 || !fold_p_update(g, a.tps, a.bs, a.order))) return cudaErrorInvalidValue;
   if (nlaunch) *nlaunch += 1;
   switch (a.prec) {
     case LQCD_FP64:

@@ -175,7 +175,17 @@ struct DslashArgs {
   double* partials = nullptr;     // one per block
   unsigned* ticket = nullptr;     // null: the sum is left as per-block partials (the solver's A-apply)
   bool pdl = false;              // programmatic dependent launch (inside captured solve graphs)
+  // The p update folded into the iteration's Dslash pair (fold_p_update): in and aux are the p before it.  The plain
+  // launch takes r + beta in at every neighbour, beta from the n_rr partials of |r|^2, and runs the beta step in an
+  // extra block; the A-apply takes r + beta aux at its own site and stores it in aux.
+  const void* upd_r = nullptr;
+  SolverDev* sd = nullptr;
+  const double* rr_partials = nullptr;
+  int n_rr = 0;
 };
+// whether launch_dslash (one system, these options) and launch_df_dslash take the p update
+bool fold_p_update(const Geom& g, int tps, int bs, int order);
+bool fold_df_p_update(const Geom& g);
 cudaError_t launch_dslash(const Geom& g, const GaugeCopies& gc, const DslashArgs& a, cudaStream_t st, int* nlaunch);
 // the same hop on 2..kMaxRhs systems sharing the operator, each link loaded once (FP32 Krylov modes, one
 // thread per site): per system the results of launch_dslash with tps = 1, bit for bit
@@ -238,6 +248,11 @@ struct DfArgs {
   const int* done = nullptr;        // if non-null and *done, the kernel returns at entry
   const int* halt = nullptr;        // likewise (the end of the double-FP32 phase of a mixed solve)
   int out_parity = 0;
+  // the p update folded in (as DslashArgs; r: hi then lo); the A-apply stores p in x
+  const float2* upd_r = nullptr;
+  SolverDev* sd = nullptr;
+  const double* rr_partials = nullptr;
+  int n_rr = 0;
 };
 // double-FP32 vectors of the LQCD_DF64 solve: [3][Vh] float2 hi, then [3][Vh] float2 lo
 struct DfUpdArgs {

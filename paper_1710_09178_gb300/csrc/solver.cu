@@ -1,7 +1,8 @@
 // solver.cu - shifted conjugate gradient on the GPU (Section 4, ref. [mcg]) with
 // mixed-precision storage, reliable updates and per-shift refinement.
 //
-// One base iteration is four kernels, all enqueued without host round trips:
+// One base iteration is four kernels (on small lattices three, with the fourth folded into the next iteration), all
+// enqueued without host round trips:
 //   1. tmp = D_oe p                                          (dslash.cu)
 //   2. q = (4m^2 + sigma_0) p - D_eo tmp, per-block partials of (p, q)   (dslash.cu epilogue)
 //   3. alpha from those partials, r -= alpha q, R[m] = r, partials of (r, r);
@@ -883,14 +884,15 @@ static DfBufs df_bufs(Workspace* w, bool phase) {
   return DfBufs{w->r, w->p, w->q, w->tmp, w->ring, w->sbytes, w->pk, nullptr};
 }
 
-// the four kernels of one base iteration
-static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase);
+// The kernels of one base iteration, number it of a window of n shifts.  On small lattices of one system the p update of
+// every iteration but the window's last is folded into the next one's Dslash pair.
+static cudaError_t enqueue_iteration_df(Launcher& L, int n, int it, bool phase);
 
-static cudaError_t enqueue_iteration(Launcher& L, int n) {
+static cudaError_t enqueue_iteration(Launcher& L, int n, int it) {
   Workspace* w = L.w;
   lqcd_ctx* ctx = L.ctx;
   cudaStream_t st = w->st;
-  if (w->kprec == LQCD_DF64) return enqueue_iteration_df(L, n, false);
+  if (w->kprec == LQCD_DF64) return enqueue_iteration_df(L, n, it, false);
   const int S = L.S;
   PerSys<DslashArgs> d1, d2;
   PerSys<RUpdArgs> ra;
@@ -903,6 +905,7 @@ static cudaError_t enqueue_iteration(Launcher& L, int n) {
   const int bs = S == 1 ? ctx->dslash_bs : 128;
   const int order = S == 1 ? ctx->dslash_order : 0;
   const int nb = (L.g.vh + 255) / 256;  // streaming blocks; one more runs the scalar step
+  const bool fold = S == 1 && w->kprec != LQCD_FP64 && fold_p_update(L.g, tps, bs, order);
   for (int s = 0; s < S; ++s) {
     Workspace* y = L.sys(s);
     DslashArgs& a = d1.s[s];
@@ -914,6 +917,12 @@ static cudaError_t enqueue_iteration(Launcher& L, int n) {
     a.bs = bs;
     a.order = order;
     a.done = &y->sd->done;
+    if (fold && it > 0) {
+      a.upd_r = y->r;
+      a.sd = y->sd;
+      a.rr_partials = y->partials_b;
+      a.n_rr = nb;
+    }
     DslashArgs& b = d2.s[s];
     b = a;
     b.out = y->q;
@@ -960,7 +969,7 @@ static cudaError_t enqueue_iteration(Launcher& L, int n) {
   else if (w->sfmt == kS16) e = launch_k(pr, r_update_kernel<float, kS16>, rgrid, dim3(256), st, L.g, ra);
   else e = launch_k(pr, r_update_kernel<float, kS32>, rgrid, dim3(256), st, L.g, ra);
   L.nlaunch += 1;
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || (fold && it < kWindow - 1)) return e;
   const bool pp = L.next_pdl();
   if (w->kprec == LQCD_FP64) e = launch_k(pp, p_update_kernel<double>, grid, dim3(256), st, L.g, pa);
   else e = launch_k(pp, p_update_kernel<float>, grid, dim3(256), st, L.g, pa);
@@ -970,7 +979,7 @@ static cudaError_t enqueue_iteration(Launcher& L, int n) {
 
 // the four kernels of one base iteration of the double-FP32 solve (LQCD_DF64, or the double-FP32
 // phase of a mixed solve)
-static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase) {
+static cudaError_t enqueue_iteration_df(Launcher& L, int n, int it, bool phase) {
   Workspace* w = L.w;
   lqcd_ctx* ctx = L.ctx;
   cudaStream_t st = w->st;
@@ -981,6 +990,7 @@ static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase) {
   PerSys<DfArgs> d, a;
   PerSys<DfUpdArgs> u;
   memset(&u, 0, sizeof(u));
+  const bool fold = S == 1 && fold_df_p_update(L.g);
   for (int s = 0; s < S; ++s) {
     Workspace* y = L.sys(s);
     const DfBufs B = df_bufs(y, phase);
@@ -994,6 +1004,12 @@ static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase) {
     x.done = &y->sd->done;
     x.halt = B.halt;
     x.out_parity = 1;
+    if (fold && it > 0) {
+      x.upd_r = hi(B.r);
+      x.sd = y->sd;
+      x.rr_partials = y->partials_b;
+      x.n_rr = (L.g.vh + 255) / 256;  // the r update's blocks
+    }
     DfArgs& z = a.s[s];
     z = x;
     z.in_hi = hi(B.tmp);
@@ -1026,7 +1042,7 @@ static cudaError_t enqueue_iteration_df(Launcher& L, int n, bool phase) {
   if (e != cudaSuccess) return e;
   e = launch_df_r_update(L.g, u, n, S, st, L.next_pdl());
   L.nlaunch += 1;
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || (fold && it < kWindow - 1)) return e;
   e = launch_df_p_update(L.g, u, S, st, L.next_pdl());
   L.nlaunch += 1;
   return e;
@@ -1253,7 +1269,7 @@ static cudaError_t enqueue_df_window(Launcher& L, int n, cudaGraphConditionalHan
   const int S = L.S;
   cudaError_t e;
   for (int it = 0; it < kWindow; ++it)
-    if ((e = enqueue_iteration_df(L, n, true)) != cudaSuccess) return e;
+    if ((e = enqueue_iteration_df(L, n, it, true)) != cudaSuccess) return e;
   if ((e = enqueue_flush(L, n, true)) != cudaSuccess) return e;
   loop_ctl_df_kernel<<<1, 32, 0, w->st>>>(handle, solver_states(L), S, set_cond);
   L.nlaunch += 1;
@@ -1292,7 +1308,7 @@ static cudaError_t enqueue_batch(Launcher& L, int n, int k0, double sigma0, int 
   const int S = L.S;
   for (int wdx = 0; wdx < windows; ++wdx) {
     for (int it = 0; it < kWindow; ++it)
-      if ((e = enqueue_iteration(L, n)) != cudaSuccess) return e;
+      if ((e = enqueue_iteration(L, n, it)) != cudaSuccess) return e;
     if ((e = enqueue_flush(L, n)) != cudaSuccess) return e;
     if (use_ru && w->df) {
       // r = fl32(b - (A + sigma_0) x_0) in double-FP32 straight into the Krylov residual
