@@ -436,6 +436,8 @@ __global__ void window_scalars_kernel(const __grid_constant__ PerSys<SolverDev*>
 // is done, or the window budget is spent); in a captured graph this ends the phase's while loop.
 __global__ void loop_ctl_df_kernel(cudaGraphConditionalHandle handle, const __grid_constant__ PerSys<SolverDev*> sds,
                                    int S, int set_cond) {
+  pdl_wait();
+  pdl_trigger();
   if (threadIdx.x != 0) return;
   // a window ran while any system was still in the phase (the systems run in lock step); each system
   // ends its own phase, the loop ends with the last
@@ -468,7 +470,7 @@ struct DemoteArgs {
   const SolverDev* sd;
 };
 
-// The change of phase, once (after the window that ended the double-FP32 phase): r, p and the active
+// The change of phase, once, after the double-FP32 phase: r, p and the active
 // shifts' p_k to the FP32 phase's storage, each the (hi, lo) pair rounded to FP32 (its hi part).
 template <int SF>
 __global__ void __launch_bounds__(256) demote_kernel(Geom g, const __grid_constant__ PerSys<DemoteArgs> pa) {
@@ -513,18 +515,13 @@ __global__ void ru_finish_kernel(Geom g, const double2* __restrict__ r64, void* 
     w.y = (T)v.y;
     static_cast<V2*>(r)[i] = w;
   }
-  // ru_skip is cleared only by ru_close_kernel, which runs after this kernel: every block sees one value
+  // ru_skip is set only by window_end_kernel, which runs after this kernel: every block sees one value
 }
 
-// bookkeeping of a reliable update, one thread, after ru_finish_kernel
-__global__ void ru_close_kernel(const __grid_constant__ PerSys<SolverDev*> sds, const __grid_constant__ PerSys<int*> counts) {
-  pdl_wait();
-  pdl_trigger();
-  if (threadIdx.x != 0) return;
-  SolverDev* sd = sds.s[blockIdx.y];
-  int* ru_count = counts.s[blockIdx.y];
+// bookkeeping of a reliable update, one thread
+__device__ __forceinline__ void ru_close(SolverDev* sd, int* ru_count) {
   if (sd->ru_skip) return;
-  double rr = sd->scal[0];
+  const double rr = sd->scal[0];
   if (!isfinite(rr)) {
     sd->status = LQCD_ERR_NONFINITE;
     sd->done = 1;
@@ -537,10 +534,17 @@ __global__ void ru_close_kernel(const __grid_constant__ PerSys<SolverDev*> sds, 
   *ru_count += 1;
 }
 
-// End of a window inside the graph's while loop: continue while the solve is running.  The
-// window counter bounds the loop by itself, whatever state the other kernels left.
-__global__ void loop_ctl_kernel(cudaGraphConditionalHandle handle, const __grid_constant__ PerSys<SolverDev*> sds, int S) {
+// End of a window of S systems: the reliable updates' bookkeeping (use_ru) and, inside the graph's while loop (loop),
+// its condition: continue while a solve is running.  The window counter bounds the loop by itself, whatever state the
+// other kernels left.
+__global__ void window_end_kernel(cudaGraphConditionalHandle handle, const __grid_constant__ PerSys<SolverDev*> sds,
+                                  const __grid_constant__ PerSys<int*> counts, int S, int use_ru, int loop) {
+  pdl_wait();
+  pdl_trigger();
   if (threadIdx.x != 0) return;
+  if (use_ru)
+    for (int y = 0; y < S; ++y) ru_close(sds.s[y], counts.s[y]);
+  if (!loop) return;
   const int wr = sds.s[0]->windows_run + 1;
   unsigned cont = 0u;
   for (int y = 0; y < S; ++y) {
@@ -1262,18 +1266,22 @@ static cudaError_t enqueue_resid_df_slots(Launcher& L, const ResidTarget* t, con
   return e;
 }
 
-// one window of the double-FP32 phase of the precision schedule, its phase test and the (guarded,
-// one-time) change to the FP32 phase
+// one window of the double-FP32 phase of the precision schedule and its phase test
 static cudaError_t enqueue_df_window(Launcher& L, int n, cudaGraphConditionalHandle handle, int set_cond) {
   Workspace* w = L.w;
-  const int S = L.S;
   cudaError_t e;
   for (int it = 0; it < kWindow; ++it)
     if ((e = enqueue_iteration_df(L, n, it, true)) != cudaSuccess) return e;
   if ((e = enqueue_flush(L, n, true)) != cudaSuccess) return e;
-  loop_ctl_df_kernel<<<1, 32, 0, w->st>>>(handle, solver_states(L), S, set_cond);
   L.nlaunch += 1;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return launch_k(L.next_pdl(), loop_ctl_df_kernel, dim3(1), dim3(32), w->st, handle, solver_states(L), L.S, set_cond);
+}
+
+// The change from the double-FP32 to the FP32 phase, once between the two loops: as a graph's nodes behind *prev (its
+// last node on return), or launched (graph null).
+static cudaError_t enqueue_demote(Launcher& L, int n, cudaGraph_t graph, cudaGraphNode_t* prev) {
+  Workspace* w = L.w;
+  const int S = L.S;
   PerSys<DemoteArgs> da;
   memset(&da, 0, sizeof(da));
   for (int s = 0; s < S; ++s) {
@@ -1291,18 +1299,35 @@ static cudaError_t enqueue_df_window(Launcher& L, int n, cudaGraphConditionalHan
     x.sd = y->sd;
   }
   const dim3 grid((L.g.vh + 255) / 256, S);
-  if (w->sfmt == kS16) e = launch_k(L.next_pdl(), demote_kernel<kS16>, grid, dim3(256), w->st, L.g, da);
-  else e = launch_k(L.next_pdl(), demote_kernel<kS32>, grid, dim3(256), w->st, L.g, da);
-  L.nlaunch += 1;
+  PerSys<SolverDev*> sds = solver_states(L);
+  if (!graph) {
+    if (w->sfmt == kS16) demote_kernel<kS16><<<grid, 256, 0, w->st>>>(L.g, da);
+    else demote_kernel<kS32><<<grid, 256, 0, w->st>>>(L.g, da);
+    demoted_kernel<<<dim3(1, S), 32, 0, w->st>>>(sds);
+    return cudaGetLastError();
+  }
+  void* args1[] = {&L.g, &da};
+  cudaKernelNodeParams k = {};
+  k.func = w->sfmt == kS16 ? reinterpret_cast<void*>(demote_kernel<kS16>) : reinterpret_cast<void*>(demote_kernel<kS32>);
+  k.gridDim = grid;
+  k.blockDim = dim3(256);
+  k.kernelParams = args1;
+  cudaGraphNode_t node;
+  cudaError_t e = cudaGraphAddKernelNode(&node, graph, prev, 1, &k);
   if (e != cudaSuccess) return e;
-  demoted_kernel<<<dim3(1, S), 32, 0, w->st>>>(solver_states(L));
-  L.nlaunch += 1;
-  return cudaGetLastError();
+  void* args2[] = {&sds};
+  k.func = reinterpret_cast<void*>(demoted_kernel);
+  k.gridDim = dim3(1, S);
+  k.blockDim = dim3(32);
+  k.kernelParams = args2;
+  return cudaGraphAddKernelNode(prev, graph, &node, 1, &k);
 }
 
 // iteration batch: windows x (kWindow iterations, flush, reliable update if due).  The reliable-update
 // kernels return at entry unless the beta step marked one as due (ru_skip == 0).
-static cudaError_t enqueue_batch(Launcher& L, int n, int k0, double sigma0, int windows, bool use_ru) {
+// loop: the while loop's condition to set at the end of the (single) window, null outside a graph.
+static cudaError_t enqueue_batch(Launcher& L, int n, int k0, double sigma0, int windows, bool use_ru,
+                                 const cudaGraphConditionalHandle* loop) {
   cudaError_t e;
   Workspace* w = L.w;
   const int S = L.S;
@@ -1310,41 +1335,39 @@ static cudaError_t enqueue_batch(Launcher& L, int n, int k0, double sigma0, int 
     for (int it = 0; it < kWindow; ++it)
       if ((e = enqueue_iteration(L, n, it)) != cudaSuccess) return e;
     if ((e = enqueue_flush(L, n)) != cudaSuccess) return e;
+    PerSys<int*> counts;
+    memset(&counts, 0, sizeof(counts));
+    for (int s = 0; s < S; ++s) counts.s[s] = L.sys(s)->ru_count;
     if (use_ru && w->df) {
       // r = fl32(b - (A + sigma_0) x_0) in double-FP32 straight into the Krylov residual
       ResidTarget t[kMaxRhs];
-      PerSys<int*> counts;
-      memset(&counts, 0, sizeof(counts));
       for (int s = 0; s < S; ++s) {
         Workspace* y = L.sys(s);
         t[s] = ResidTarget{run_solutions(y)[k0], static_cast<float2*>(y->r), &y->sd->scal[0], &y->sd->ru_skip};
-        counts.s[s] = y->ru_count;
       }
       if ((e = enqueue_resid_df(L, t, sigma0, true)) != cudaSuccess) return e;
-      if ((e = launch_k(L.next_pdl(), ru_close_kernel, dim3(1, S), dim3(32), w->st, solver_states(L), counts)) !=
-          cudaSuccess)
-        return e;
-      L.nlaunch += 1;
     } else if (use_ru) {
       // one system: r64 = b - (A + sigma_0) x_0 in FP64 with FP64 links, then r <- r64, |r|^2 <- |r64|^2
       if ((e = enqueue_resid64(L, w->xk[k0], w->b64, sigma0, &w->sd->scal[0], &w->sd->ru_skip, &w->sd->a_diag)) !=
           cudaSuccess)
         return e;
       int nb3 = (3 * L.g.vh + 255) / 256;
-      const bool pf = L.next_pdl(), pc = L.next_pdl();
+      const bool pf = L.next_pdl();
       const double2* r64 = w->r64;
       const SolverDev* sdc = w->sd;
       if (w->kprec == LQCD_FP64)
         e = launch_k(pf, ru_finish_kernel<double>, dim3(nb3), dim3(256), w->st, L.g, r64, w->r, sdc);
       else
         e = launch_k(pf, ru_finish_kernel<float>, dim3(nb3), dim3(256), w->st, L.g, r64, w->r, sdc);
-      PerSys<int*> counts;
-      memset(&counts, 0, sizeof(counts));
-      counts.s[0] = w->ru_count;
-      if (e == cudaSuccess)
-        e = launch_k(pc, ru_close_kernel, dim3(1, 1), dim3(32), w->st, solver_states(L), counts);
-      L.nlaunch += 2;
+      L.nlaunch += 1;
       if (e != cudaSuccess) return e;
+    }
+    if (use_ru || loop) {
+      const cudaGraphConditionalHandle h = loop ? *loop : 0;
+      L.nlaunch += 1;
+      if ((e = launch_k(L.next_pdl(), window_end_kernel, dim3(1), dim3(32), w->st, h, solver_states(L), counts, S,
+                        use_ru ? 1 : 0, loop ? 1 : 0)) != cudaSuccess)
+        return e;
     }
   }
   return cudaSuccess;
@@ -1442,6 +1465,7 @@ static int solve_core(Launcher& L, const double* shifts, int n, double tol, int 
           cudaError_t e1 = cudaStreamEndCapture(w->st, &captured1);
           if (e == cudaSuccess) e = e1;
           nodes_df = C1.nlaunch;
+          if (e == cudaSuccess) e = enqueue_demote(L, n, graph, &prev);
         }
         cudaGraphConditionalHandle handle;
         LQ_CUDA(cudaGraphConditionalHandleCreate(&handle, graph, 1, cudaGraphCondAssignDefault));
@@ -1458,12 +1482,7 @@ static int solve_core(Launcher& L, const double* shifts, int n, double tol, int 
         C.pdl = pdl;
         C.chained = false;
         LQ_CUDA(cudaStreamBeginCaptureToGraph(w->st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        if (e == cudaSuccess) e = enqueue_batch(C, n, k0, sigma0, 1, use_ru);
-        if (e == cudaSuccess) {
-          loop_ctl_kernel<<<1, 32, 0, w->st>>>(handle, solver_states(C), S);
-          C.nlaunch += 1;
-          e = cudaGetLastError();
-        }
+        if (e == cudaSuccess) e = enqueue_batch(C, n, k0, sigma0, 1, use_ru, &handle);
         cudaGraph_t captured;
         cudaError_t e2 = cudaStreamEndCapture(w->st, &captured);
         if (e == cudaSuccess) e = e2;
@@ -1494,7 +1513,7 @@ static int solve_core(Launcher& L, const double* shifts, int n, double tol, int 
           if (df_phase) {
             for (int wdx = 0; wdx < windows; ++wdx) LQ_CUDA(enqueue_df_window(L, n, 0, 0));
           } else {
-            LQ_CUDA(enqueue_batch(L, n, k0, sigma0, windows, use_ru));
+            LQ_CUDA(enqueue_batch(L, n, k0, sigma0, windows, use_ru, nullptr));
           }
           int slot = launched & 1;
           for (int s = 0; s < S; ++s)
@@ -1520,6 +1539,7 @@ static int solve_core(Launcher& L, const double* shifts, int n, double tol, int 
     if (sched) {
       int rc = run_batches(true);
       if (rc != LQCD_OK) return rc;
+      LQ_CUDA(enqueue_demote(L, n, nullptr, nullptr));
     }
     int rc = run_batches(false);
     if (rc != LQCD_OK) return rc;
@@ -1544,6 +1564,7 @@ static int solve_core(Launcher& L, const double* shifts, int n, double tol, int 
     int wdf = 0;
     if (sched)
       for (int s = 0; s < S; ++s) wdf = std::max(wdf, L.sys(s)->host_ints[2]);
+    if (sched) L.nlaunch += 2;  // the change of phase
     L.nlaunch += nodes_fp32 * (w->host_ints[0] - wdf) + nodes_df * wdf;
   }
   for (int s = 0; s < S; ++s) {
