@@ -9,7 +9,8 @@
 // per call) and 8 neighbour vectors (the input vector is small and stays in L2).
 // TPS threads cooperate on one site, each taking 8/TPS of the hops, and combine
 // their partial sums with warp shuffles; more threads per site means more
-// independent loads in flight per SM.
+// independent loads in flight per SM.  The FP64 mode has a kernel of its own (dslash64_kernel: products on
+// the integer multiplier), and so have lattices of at most one block per SM (AHEAD: all loads at once).
 #include <string.h>
 
 #include <algorithm>

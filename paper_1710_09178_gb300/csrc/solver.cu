@@ -9,8 +9,8 @@
 //      an extra block stores alpha (solver_dev.cuh)                      (r_update_kernel)
 //   4. beta from those partials, p = r + beta p; an extra block stores beta and
 //      decides the base stopping test and the reliable update           (p_update_kernel)
-// Every kWindow iterations the per-shift recurrences of the window are replayed from the
-// stored alpha and beta, one block per shift (window_scalars_kernel), and the window kernel
+// The per-shift recurrences follow one iteration behind from the stored alpha and beta, one block per shift beside
+// step 3; every kWindow iterations their last one is made up (window_scalars_kernel), and the window kernel
 // applies the pending x_k / p_k updates of all shifts at once (flush_kernel): each shift vector
 // is read and written once per window instead of once per iteration, which is what makes the
 // multi-shift update (the heaviest loop of the shifted CG in Section 7) cheap.  A whole solve is

@@ -87,9 +87,10 @@ __device__ __forceinline__ void init_scalars(SolverDev* sd, const InitParams& ip
 // The base iteration needs only alpha and beta; the per-shift recurrences (zeta_k, the window
 // coefficients, the stopping tests of the shifts) depend on nothing but the sequence of alpha and
 // beta.  So the two steps below store the base scalars of the iteration and decide the base
-// stopping test, and window_scalars_shift() follows with the per-shift recurrences.  The base shift stops last: for s_k >= 0, |zeta_k| <= 1 (zeta_k is the inverse of the
-// base residual polynomial at -s_k), and zeta_0 = 1 exactly, so "every shift has stopped" is "the
-// base residual has": |r_new|^2 <= tol^2 |b|^2.
+// stopping test, and window_scalars_shift() follows with the per-shift recurrences.  The base
+// shift stops last: for s_k >= 0, |zeta_k| <= 1 (zeta_k is the inverse of the base residual
+// polynomial at -s_k), and zeta_0 = 1 exactly, so "every shift has stopped" is "the base residual
+// has": |r_new|^2 <= tol^2 |b|^2.
 
 // the block that runs the step; all its threads call.  pa = (Re<p, q>, alpha = |r|^2 / Re<p, q>
 // with its FP32 and (hi, lo) copies), formed once by thread 0 of every block.
