@@ -86,6 +86,7 @@ constexpr int kFixSites = 32, kFixThreads = 4 * kFixSites;
 
 struct FixShared {
   longlong2 part[4][3][kFixSites];
+  int2 fwd[4][3][kFixSites];  // upper words of the forward hops' sums (fix_hop_words)
   int word[4][kFixSites];
 };
 
@@ -128,6 +129,8 @@ struct FixGroup {
       s.rx[c] = s.ix[c] = 1 << (kFixLow - 1);  // rounds the shift below
     }
     fix_hop<true>(s, Lf, vf, E);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sh.fwd[mu][c][ls] = make_int2(fix_upper(s.rh[c]), fix_upper(s.ih[c]));
     fix_hop<false>(s, Lb, vb, E);
     const bool bad = Lf.e[0].x == kFixBadLink || Lb.e[0].x == kFixBadLink;
 #pragma unroll
@@ -149,15 +152,23 @@ struct FixGroup {
     int64_t re = 0, im = 0;
     bool ok = false;
     if (U) {
-      E = exponent(sh, ls);
+      const int w[4] = {sh.word[0][ls], sh.word[1][ls], sh.word[2][ls], sh.word[3][ls]};
+      E = fix_block_exponent(w);
       ok = E >= 0;
+      uint32_t hr = 0, hi = 0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const longlong2 u = sh.part[q][c][ls];
+        const int2 f = sh.fwd[q][c][ls];
         ok = ok && u.x != kFixBadSum;
         re += u.x;
         im += u.y;
+        hr += fix_hop_words(f.x, fix_upper(u.x));
+        hi += fix_hop_words(f.y, fix_upper(u.y));
       }
+      const bool zero = (w[0] | w[1] | w[2] | w[3]) == 0;  // all neighbours
+      const uint32_t need = fix_needed(w, E);
+      ok = ok && (zero || (hr >= need && hi >= need));
     }
     if (!ok) {
       const Vec3<double> d = site64_fma(g, U64, in, p, i);

@@ -12,16 +12,24 @@
 // an accumulator of their own, L L dropped), 864 per site: 13.5 clocks, beside about 20 shifts and logic
 // operations per component for the digits.  With one exponent per output site all products add up as
 // integers, so the sum does not depend on its order, and one conversion per component rounds it to FP64.
-// The steps before that rounding err by about 2^-57 of the largest neighbour's component, less than each of
-// the 48 roundings of an FP64 sum: against quad precision the hop's error is 4.9e-17, that of the FP64
-// multiply-adds 1.7e-16 (Gaussian vectors, 8 x 6 x 4 x 6).
+//
+// Accuracy.  With 2^E the power of two at or below the largest neighbouring component and m_mu 2^E the largest one of
+// direction mu's two neighbours, the steps before that rounding err per real component by at most 2^(E-58) times
+// 12 sum_mu m_mu (links rounded to 2^-58), 20 (vectors truncated at 2^(E-57) against rows of norm 1/2), 48 (48 dropped
+// L L products) and 2 (the H L sums rounded once per direction).  What counts for the result is S, the sum of
+// the magnitudes of the component's own 48 products, which may be far smaller: links that do not mix the
+// colours beside colours of different size, or entries below 2^-57 of their unit.  The digits are used where that
+// error is below 21 x 2^-53 S, that of the 25 roundings of an FP64 multiply-add chain; S is bounded from below by the
+// eight hops' magnitudes (fix_hop_words, fix_needed).  A component short of it is computed in FP64: on rough fields with
+// Gaussian vectors (S of 5 to 10 2^E, 0.1 to 0.26 2^E needed) one in about 2 million.  Against quad precision the
+// hop's error is 4.9e-17, that of the FP64 multiply-adds 1.7e-16 (Gaussian vectors, 8 x 6 x 4 x 6).
 //
 // The integers' ranges.  A row or column of 1/2 U has norm 1/2; the format takes up to kFixMaxNorm = 0.501, so
 // that by the Cauchy-Schwarz inequality every partial sum of a component's 48 products is at most
 // 8 x 0.501 x sqrt(6) = 9.82 times 2^29 2^30 in units of H H: 2^62.3.  The 24 H L products of one thread's two
 // hops are at most 12 2^28 (2^30 + 2^28.1) < 2^62.
 //
-// What does not fit (a link with a row or column of larger norm or not finite, neighbours whose largest
+// What else does not fit (a link with a row or column of larger norm or not finite, neighbours whose largest
 // component lies outside 2^-800 .. 2^800 or is not finite) marks the site, which is then computed in FP64.
 //
 // Plain integer arithmetic: the host build, used by the tests, gives the device's bits.
@@ -165,6 +173,22 @@ LQCD_FIX_HD int fix_block_exponent(const int (&w)[N]) {
   }
   const int E = m >> 20;
   return any < 0 || E > kFixMaxE ? -1 : (E < kFixMinE ? kFixMinE : E);
+}
+
+// The least sum over the eight hops of the magnitudes of their sums' upper 32 bits (fix_hop_words) with which a
+// component's digits are accurate enough: (70 + 12 sum_mu m_mu) 2^-58 <= 21 x 2^-53 S / 2^E, S / 2^E = words 2^-26, so
+// words >= (70 + 12 sum m) 2^26 / 672; here 2^20 (7 + 1.25 sum m), more than 4 % above it, which takes what the
+// upper words leave out.  w: the max words of the four directions.
+LQCD_FIX_HD uint32_t fix_needed(const int (&w)[4], int E) {
+  uint32_t m = 0;
+  for (int q = 0; q < 4; ++q) m += fix_shr32(1u << 20 | ((uint32_t)w[q] & 0xfffffu), E - (w[q] >> 20));
+  return (7u << 20) + m + (m >> 2);
+}
+LQCD_FIX_HD int fix_upper(int64_t sum) { return (int)(sum >> 32); }
+// |a hop's sum| is at most its products' magnitudes together.  fwd, both: upper words after the forward hop and both
+LQCD_FIX_HD uint32_t fix_hop_words(int fwd, int both) {
+  const uint32_t f = (uint32_t)fwd, b = (uint32_t)both - f;
+  return (fwd < 0 ? 0u - f : f) + ((int)b < 0 ? 0u - b : b);
 }
 
 // hh += the H H product, x += the two H L products of (ah, al) and b
