@@ -162,12 +162,21 @@ static __device__ __noinline__ M3 link_times_staples(Geom g, const double2* __re
 }
 
 // The same products in fixed point (fixpoint.h), from the digits of 1/2 eta bc U.  A matrix is (re.h, re.l,
-// im.h, im.l) per entry, F = H 2^28 + L with L >= 0 here; a product's entries are 64-bit sums in units of 2^56 of
-// the product of the factors' units, whose digits (fix_split) are the next product's factor:
-//   folded links in units of 2^-57, entries <= 1/2;   U U in 2^-58, <= 1/4;   U U U in 2^-59, <= 1/8;
-//   the six staples' sum, divided by 4, in 2^-57, <= 3/4;   U A in 2^-58, <= 3/8.
-// The H H sums stay below 6 2^28 2^28.6 = 2^59.2, the H L sums below 6 (2^28 2^28 + 2^28 2^28.6) = 2^60; each product
-// drops and rounds less than 8 units, 2^-55 of 1/4.
+// im.h, im.l) per entry, F = H 2^28 + L (links: H and L of one sign; split products: 0 <= L < 2^28); a product's
+// entries are 64-bit sums in units of 2^56 of the product of the factors' units, whose digits (fix_split) are the
+// next product's factor:
+//   folded links in units of 2^-57, entries <= 1/2;   U U in 2^-58, <= 1/4;   U U U in 2^-59, <= 0.22;
+//   the six staples' sum, divided by 4, in 2^-57, <= 0.33;   U A in 2^-58, <= 1.6.
+// The H H sums stay below 6 2^28 2^29.4, the H L sums below 6 (2^28 2^28 + 2^28 2^29.4).
+//
+// Accuracy, with u = 2^-58 and rows and columns of norm up to kFixMaxNorm, so that the six components of a row add up to
+// 1.23 at most.  Links are rounded by u.  A product of links errs by 2 x 1.23 u from that, 6 u from the L L products and
+// u/2 from rounding: 9 u; times a link: 9 x 1.23 + 1.1 + 3 + 0.25 = 15.3 u; the six staples' sum: 93 u; times the link:
+// 93 x 1.23 + 5.6 + 6.5 = 126 u.  W is 16 times that: 63 x 2^-53, whatever the size of the component.  The FP64 products
+// err by at most 24 x 2^-53 S (three products of 6 roundings each and six sums), S the sum of the magnitudes of all products of
+// links that make up the component.  So the digits' W is taken where S > 63 / 24, S bounded from below by |U| sum |UU| |U|
+// in FP32 (staple_magnitude), for each combination of components that the force is made of; a link short of that is
+// computed in FP64 (fields close to one, whose off-diagonal and imaginary parts are small).
 struct FixSum3 {
   int64_t re[9], im[9];
 };
@@ -213,13 +222,74 @@ __device__ __forceinline__ FixLink fix_split(const FixSum3& s, int shift) {  // 
   return o;
 }
 
+// mag += |op(A)| |op(B)| (real and imaginary parts of each entry: the sums of the magnitudes of their products), from the
+// high digits: in units of theirs, and below the true magnitudes but for 2^-22 of them.
+constexpr int kForceThreads = 128;
+typedef float ForceMag[18][kForceThreads];  // [entry, re and im][thread]
+template <bool AD, bool BD>
+__device__ __forceinline__ void staple_magnitude(ForceMag& mag, const FixLink& A, const FixLink& B) {
+  float a[18], b[18];
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    a[2 * j] = fabsf((float)A.e[j].x);
+    a[2 * j + 1] = fabsf((float)A.e[j].z);
+    b[2 * j] = fabsf((float)B.e[j].x);
+    b[2 * j + 1] = fabsf((float)B.e[j].z);
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      float re = 0.f, im = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int ja = 2 * (AD ? 3 * k + r : 3 * r + k), jb = 2 * (BD ? 3 * q + k : 3 * k + q);
+        re = fmaf(a[ja], b[jb], fmaf(a[ja + 1], b[jb + 1], re));
+        im = fmaf(a[ja], b[jb + 1], fmaf(a[ja + 1], b[jb], im));
+      }
+      mag[2 * (3 * r + q)][threadIdx.x] += re;
+      mag[2 * (3 * r + q) + 1][threadIdx.x] += im;
+    }
+}
+
+// Whether |U| mag is large enough for the digits' W, for the combinations that the force takes: W_rc - conj(W_cr), the
+// differences of the diagonal's imaginary parts.
+__device__ __forceinline__ bool force_accurate(const FixLink& U, const ForceMag& mag) {
+  float u[18];
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    u[2 * j] = fabsf((float)U.e[j].x);
+    u[2 * j + 1] = fabsf((float)U.e[j].z);
+  }
+  auto S = [&](int r, int c, bool imag) {
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int ju = 2 * (3 * r + k), jm = 2 * (3 * k + c);
+      s = fmaf(u[ju], mag[jm + imag][threadIdx.x], fmaf(u[ju + 1], mag[jm + !imag][threadIdx.x], s));
+    }
+    return s;
+  };
+  // magnitudes in units of 2^-29 (link) 2^-30 (U U) 2^-29 (link) of W / 16
+  constexpr float need = 2.7f * 0x1p84f;  // 63 / 24 and what the high digits and FP32 leave out
+  bool ok = true;
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int c = r + 1; c < 3; ++c)
+      ok = ok && S(r, c, false) + S(c, r, false) >= 2 * need && S(r, c, true) + S(c, r, true) >= 2 * need;
+  const float d0 = S(0, 0, true), d1 = S(1, 1, true), d2 = S(2, 2, true);
+  return ok && d0 + d1 >= 2 * need && d0 + d1 + 2 * d2 >= 4 * need;
+}
+
 // F[l][mu][a] += beta-scaled gauge force components tr(lambda^a F_g); block: 32 sites of one parity, one direction
 // per warp.  The 13 matrix products of a link in FP64 take 1404 multiply-adds, 702 clocks of the SM's FP64 pipe; in
 // fixed point 4212 integer ones, 66 clocks, and about as much again for digits and addresses: 24^3 x 6 (331 776
 // links) 1865 -> 320 us.  Links outside the format, or no digits (Ufix null): FP64.
-__global__ void __launch_bounds__(128, 2) gauge_force_kernel(Geom g, const double2* __restrict__ U,
-                                                             const int4* __restrict__ Ufix, double beta,
-                                                             double* __restrict__ F) {
+__global__ void __launch_bounds__(kForceThreads, 2) gauge_force_kernel(Geom g, const double2* __restrict__ U,
+                                                                       const int4* __restrict__ Ufix, double beta,
+                                                                       double* __restrict__ F) {
+  __shared__ ForceMag mag;  // each thread's own column
   const int vh = g.vh;
   const int nb = (vh + 31) / 32;
   const int p = (int)blockIdx.x >= nb ? 1 : 0;
@@ -239,7 +309,10 @@ __global__ void __launch_bounds__(128, 2) gauge_force_kernel(Geom g, const doubl
     };
     FixSum3 A;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) A.re[j] = A.im[j] = 2;  // rounds the division by 4 below
+    for (int j = 0; j < 9; ++j) {
+      A.re[j] = A.im[j] = 2;  // rounds the division by 4 below
+      mag[2 * j][threadIdx.x] = mag[2 * j + 1][threadIdx.x] = 0.f;
+    }
 #pragma unroll 1
     for (int m = 1; m < 4; ++m) {
       const int nu = (mu + m) & 3;
@@ -247,17 +320,23 @@ __global__ void __launch_bounds__(128, 2) gauge_force_kernel(Geom g, const doubl
       const int xmnu = neighbour_addr(g, neighbour_bwd(g, s, nu));
       const int xpmu_mnu = neighbour_addr(g, neighbour_bwd(g, sp, nu));
       const FixLink up2 = fix_split(fix_mm<false, true>(link(1 - p, nu, xpmu), link(1 - p, mu, xpnu)), 0);
-      const FixSum3 up = fix_mm<false, true>(up2, link(p, nu, s.l));
+      const FixLink un = link(p, nu, s.l);
+      const FixSum3 up = fix_mm<false, true>(up2, un);
+      staple_magnitude<false, true>(mag, up2, un);
       // (U_mu(x-nu) U_nu(x+mu-nu))^+ U_nu(x-nu)
       const FixLink dn2 = fix_split(fix_mm<false, false>(link(1 - p, mu, xmnu), link(p, nu, xpmu_mnu)), 0);
-      const FixSum3 dn = fix_mm<true, false>(dn2, link(1 - p, nu, xmnu));
+      const FixLink um = link(1 - p, nu, xmnu);
+      const FixSum3 dn = fix_mm<true, false>(dn2, um);
+      staple_magnitude<true, false>(mag, dn2, um);
 #pragma unroll
       for (int j = 0; j < 9; ++j) {
         A.re[j] += up.re[j] + dn.re[j];
         A.im[j] += up.im[j] + dn.im[j];
       }
     }
-    const FixSum3 W = fix_mm<false, false>(link(p, mu, s.l), fix_split(A, 2));
+    const FixLink ul = link(p, mu, s.l);
+    ok = ok && force_accurate(ul, mag);
+    const FixSum3 W = fix_mm<false, false>(ul, fix_split(A, 2));
     // the links' factors 1/2 and eta bc: 1/16, and the staggered signs around a plaquette multiply to -1
     const double sc = -16.0 * 0x1p-58;
 #pragma unroll
