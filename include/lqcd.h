@@ -105,7 +105,8 @@ int lqcd_set_stream(lqcd_ctx* ctx, void* stream);
  * Builds the internal copies (FP64 and FP32 with 1/2 eta_mu and the boundary sign
  * folded in; FP32 12-real rows 0-1 without signs; the compressed forms of Section 5's outlook,
  * without signs: 8-real FP32 and 16-bit rows 0-1).  The 12-real, 8-real and 16-bit forms
- * assume the links are in SU(3).  8-real form, rows a, b, c: [a2, a3 | b1, arg a1, arg c1]
+ * assume the links are in SU(3).  The copies take 1572 bytes per site, and 576 more with the FP64
+ * links' fixed-point digits (LQCD_OPT_FP64_DIGITS).  8-real form, rows a, b, c: [a2, a3 | b1, arg a1, arg c1]
  * with a1 = sqrt(1-N) e^{i arg a1}, N = |a2|^2 + |a3|^2, c1 = sqrt(N - |b1|^2) e^{i arg c1},
  * and b2, b3, c2, c3 from the orthogonality of the rows and c = conj(a x b); links with
  * N < 1e-14 are block-diagonal and store [b2, b3 | 0, arg a1, 8].  16-bit form: int16 codes
@@ -251,6 +252,10 @@ int lqcd_neighbour_table(lqcd_ctx* ctx, int* fwd_dev, int* bwd_dev, int* sign_de
 #define LQCD_OPT_DSLASH_ORDER 11     /* block-to-site order of the FP32 Dslash: 0 linear (default), 1 the two halves
                                         of the site range interleaved (blocks running together stream from two
                                         distant regions of the vectors and link blocks) */
+#define LQCD_OPT_FP64_DIGITS 12      /* 1 = keep the FP64 links as fixed-point digits too (576 bytes per site; faster FP64
+                                        hops, solves and gauge forces) where they take at most 1/32 of the free device
+                                        memory (default), 0 = never.  Chosen at the context's first lqcd_set_gauge
+                                        (LQCD_ERR_STATE after it).  No result depends on it */
 int lqcd_set_option(lqcd_ctx* ctx, int key, double value);
 
 /*

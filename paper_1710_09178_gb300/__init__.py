@@ -50,6 +50,7 @@ OPT_DF_RESID = 8
 OPT_DF_SWITCH = 9
 OPT_DSLASH_BS = 10
 OPT_DSLASH_ORDER = 11
+OPT_FP64_DIGITS = 12
 
 MAX_SHIFTS = 32
 MAX_BATCH = 128

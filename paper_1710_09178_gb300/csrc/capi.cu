@@ -155,19 +155,19 @@ int lqcd::set_gauge(lqcd_ctx* ctx, const double* U_dev, bool all) {
   cudaError_t e;
   size_t vh = (size_t)ctx->Vh;
   if (!gc.block) {
-    // one allocation for all copies; the digits of the FP64 Dslash last, left out where they would take more
-    // than a quarter of what is free (the Dslash works without them, slower)
-    const size_t bytes[] = {2 * 4 * 9 * vh * sizeof(double2), 2 * 4 * 18 * vh * sizeof(float),
-                            2 * 4 * 18 * vh * sizeof(float),  2 * 4 * 3 * vh * sizeof(float4),
-                            2 * 4 * 2 * vh * sizeof(float4),  2 * 4 * 24 * vh};
+    // one allocation for all copies; the digits of the FP64 links last, left out where they would take more than 1/32 of
+    // what is free (all results are the same without them)
+    const size_t bytes[] = {2 * 4 * vh * (9 * sizeof(double2) + 1), 2 * 4 * 18 * vh * sizeof(float),
+                            2 * 4 * 18 * vh * sizeof(float),        2 * 4 * 3 * vh * sizeof(float4),
+                            2 * 4 * 2 * vh * sizeof(float4),        2 * 4 * 24 * vh};
     size_t off[7] = {0};
     for (int j = 0; j < 6; ++j) off[j + 1] = (off[j] + bytes[j] + 255) / 256 * 256;
     const size_t digits = 2 * 4 * fix_block_entries(g.vh) * sizeof(int4);
-    bool fix = true;
-    if (digits > (1u << 30)) {
+    bool fix = ctx->fp64_digits != 0;
+    if (fix && digits > (64u << 20)) {
       size_t left = 0, total = 0;
       if ((e = cudaMemGetInfo(&left, &total)) != cudaSuccess) return cuda_check(ctx, e, "cudaMemGetInfo");
-      fix = left > off[6] && digits <= (left - off[6]) / 4;
+      fix = left > off[6] && digits <= (left - off[6]) / 32;
     }
     e = cudaMalloc(&gc.block, off[6] + (fix ? digits : 0));
     if (e == cudaErrorMemoryAllocation && fix) {
@@ -333,8 +333,10 @@ int dslash_eo_batch(lqcd_ctx* const* ctxs, void* const* out_devs, const void* co
     }
   }
   if (dev_tab) {
-    e = launch_dslash_batch_table(static_cast<const BatchTable*>(dev_tab), tab.chunk_end[n], prec, c0->tickets + 7,
-                                  n_sm, c0->stream);
+    bool digits = true;  // FP64: of every lattice
+    for (int l = 0; l < n; ++l) digits = digits && tab.lat[l].links;
+    e = launch_dslash_batch_table(static_cast<const BatchTable*>(dev_tab), tab.chunk_end[n], prec, digits,
+                                  c0->tickets + 7, n_sm, c0->stream);
     c0->launches += 1;
     return cuda_check(c0, e, "dslash_eo_batch");
   }
@@ -477,6 +479,10 @@ int lqcd_set_option(lqcd_ctx* ctx, int key, double value) {
     case LQCD_OPT_DSLASH_ORDER:
       if (v != 0 && v != 1) return fail(ctx, LQCD_ERR_ARG, "site order must be 0 or 1");
       ctx->dslash_order = v;
+      break;
+    case LQCD_OPT_FP64_DIGITS:
+      if (ctx->gauge.block) return fail(ctx, LQCD_ERR_STATE, "the FP64 digits are chosen before the first gauge field");
+      ctx->fp64_digits = v ? 1 : 0;
       break;
     default: return fail(ctx, LQCD_ERR_ARG, "unknown option");
   }

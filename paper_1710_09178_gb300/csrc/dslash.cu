@@ -23,7 +23,8 @@
 
 namespace lqcd {
 
-enum LinkFmt { kL64 = 0, kL32 = 1, kL12 = 2, kL8 = 3, kL16 = 4 };  // kL12 and up: signs applied after loading
+// kL12 and up: signs applied after loading; kL64N: FP64 without digits (FixField)
+enum LinkFmt { kL64N = -1, kL64 = 0, kL32 = 1, kL12 = 2, kL8 = 3, kL16 = 4 };
 
 constexpr int kSMs = 152;         // GB300
 constexpr int kFixResident = 3;  // blocks per SM of the FP64 kernels (168 registers per thread)
@@ -42,7 +43,7 @@ struct KArgs {
   double* partials;
   unsigned* ticket;
   const void* links;
-  const double2* links64;  // FP64 only: the copy behind the fixed-point one
+  const double2* links64;  // FP64 only (links: its digits or null, FixField)
   int order;  // block-to-site order (site_block)
   const void* upd_r;  // the p update folded in (DslashArgs)
   SolverDev* sd;
@@ -391,18 +392,19 @@ __global__ void __launch_bounds__(128, 1) dslash_pupdate_kernel(Geom g, KArgs k)
 
 // FP64: the products in block fixed point (fix64.cuh), one direction per thread.  Blocks take groups of
 // kFixSites sites in turn; the next group's forward links are in flight while a group is finished.
-template <int EPI>
+// DIGITS: whether the field keeps its digits (FixField); half Dslash at 32^3x8 36 us with, 50 without (FP64 multiply-adds: 70).
+template <int EPI, bool DIGITS>
 __global__ void __launch_bounds__(kFixThreads, kFixResident) dslash64_kernel(Geom g, KArgs k) {
   __shared__ FixShared sh;
   const int vh = g.vh;
   const int mu = threadIdx.x / kFixSites, ls = threadIdx.x % kFixSites;
   const int p = k.out_parity;
   const double2* in = static_cast<const double2*>(k.in);
-  const int4* U = static_cast<const int4*>(k.links);
+  const FixField U{static_cast<const int4*>(k.links), k.links64};
   const uint64_t pol = policy_evict_first();  // 8 % faster than evict_last, or than keeping part of them
   const int step = gridDim.x * kFixSites;
   int i = blockIdx.x * kFixSites + ls;
-  FixGroup grp;
+  FixGroup<DIGITS> grp;
   if (i < vh) grp.start(g, U, p, i, mu, pol);
   pdl_wait();
   pdl_trigger();
@@ -422,7 +424,7 @@ __global__ void __launch_bounds__(kFixThreads, kFixResident) dslash64_kernel(Geo
     if (i + step < vh) grp.start(g, U, p, i + step, mu, pol);
     __syncthreads();
     if (mine) {
-      const Cplx<double> d = FixGroup::colour(sh, g, U, k.links64, in, p, i, mu, ls);
+      const Cplx<double> d = FixGroup<DIGITS>::colour(sh, g, k.links64, in, p, i, mu, ls);
       double2 w = make_double2(d.re, d.im);
       if constexpr (EPI != (int)Epi::Plain) {
         w = make_double2(a * ps.x - d.re, a * ps.y - d.im);
@@ -541,20 +543,21 @@ __device__ __forceinline__ void batch_loop(const BatchLattice* lat, const int* c
     if (l >= n) continue;
     const BatchLattice& L = lat[l];
     const int i0 = (it - chunk_end[l]) * kBatchChunk;
-    if constexpr (LF == kL64) {
+    if constexpr (LF <= kL64) {
       __shared__ FixShared sh;
       const int mu = threadIdx.x / kFixSites, ls = threadIdx.x % kFixSites, vh = L.g.vh, p = L.out_parity;
-      const int4* U = static_cast<const int4*>(L.links);
+      const FixField U{static_cast<const int4*>(L.links), L.links64};
       const double2* in = static_cast<const double2*>(L.in);
+      typedef FixGroup<LF == kL64> Group;
       for (int j0 = i0; j0 < min(i0 + kBatchChunk, vh); j0 += kFixSites) {
         const int i = j0 + ls;
         const bool valid = i < vh;
-        FixGroup grp;
+        Group grp;
         if (valid) grp.start(L.g, U, p, i, mu, pol);
         grp.hops(sh, L.g, U, in, p, mu, ls, valid, pol);
         __syncthreads();
         if (valid && mu < 3) {
-          const Cplx<double> d = FixGroup::colour(sh, L.g, U, L.links64, in, p, i, mu, ls);
+          const Cplx<double> d = Group::colour(sh, L.g, L.links64, in, p, i, mu, ls);
           static_cast<double2*>(L.out)[(size_t)mu * vh + i] = make_double2(d.re, d.im);
         }
         __syncthreads();
@@ -573,7 +576,7 @@ __device__ __forceinline__ void batch_loop(const BatchLattice* lat, const int* c
 
 // descriptors in the parameter block (up to kBatchPerLaunch lattices), copied to shared memory
 template <int LF>
-__global__ void __launch_bounds__(kBatchChunk, LF == kL64 ? kFixResident : 7)
+__global__ void __launch_bounds__(kBatchChunk, LF <= kL64 ? kFixResident : 7)
     dslash_batch_kernel(BatchArgs a, unsigned* head) {
   __shared__ BatchLattice lat[kBatchPerLaunch];
   __shared__ int chunk_end[kBatchPerLaunch + 1];
@@ -592,7 +595,7 @@ __global__ void __launch_bounds__(kBatchChunk, LF == kL64 ? kFixResident : 7)
 
 // descriptors in a device table (up to kMaxBatch lattices), copied to shared memory
 template <int LF>
-__global__ void __launch_bounds__(kBatchChunk, LF == kL64 ? kFixResident : 7)
+__global__ void __launch_bounds__(kBatchChunk, LF <= kL64 ? kFixResident : 7)
     dslash_batch_table_kernel(const BatchTable* __restrict__ tab, unsigned* head) {
   __shared__ BatchLattice lat[kMaxBatch];
   __shared__ int chunk_end[kMaxBatch + 1];
@@ -615,7 +618,13 @@ cudaError_t launch_dslash_batch(const BatchArgs& a, int prec, unsigned* head, in
   // one resident wave of persistent blocks
   const unsigned grid = (unsigned)std::min(items, (prec == LQCD_FP64 ? kFixResident : 7) * n_sm);
   switch (prec) {
-    case LQCD_FP64: dslash_batch_kernel<kL64><<<grid, kBatchChunk, 0, st>>>(a, head); break;
+    case LQCD_FP64: {
+      bool digits = true;  // of every lattice
+      for (int j = 0; j < a.n; ++j) digits = digits && a.lat[j].links;
+      if (digits) dslash_batch_kernel<kL64><<<grid, kBatchChunk, 0, st>>>(a, head);
+      else dslash_batch_kernel<kL64N><<<grid, kBatchChunk, 0, st>>>(a, head);
+      break;
+    }
     case LQCD_FP32_R12: dslash_batch_kernel<kL12><<<grid, kBatchChunk, 0, st>>>(a, head); break;
     case LQCD_FP32_R8: dslash_batch_kernel<kL8><<<grid, kBatchChunk, 0, st>>>(a, head); break;
     case LQCD_FP32_L16: dslash_batch_kernel<kL16><<<grid, kBatchChunk, 0, st>>>(a, head); break;
@@ -624,7 +633,7 @@ cudaError_t launch_dslash_batch(const BatchArgs& a, int prec, unsigned* head, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_dslash_batch_table(const BatchTable* tab, int n_items, int prec, unsigned* head, int n_sm,
+cudaError_t launch_dslash_batch_table(const BatchTable* tab, int n_items, int prec, bool digits, unsigned* head, int n_sm,
                                       cudaStream_t st) {
   if (n_items <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(head, 0, sizeof(unsigned), st);
@@ -632,7 +641,10 @@ cudaError_t launch_dslash_batch_table(const BatchTable* tab, int n_items, int pr
   // one resident wave of persistent blocks
   const unsigned grid = (unsigned)std::min(n_items, (prec == LQCD_FP64 ? kFixResident : 7) * n_sm);
   switch (prec) {
-    case LQCD_FP64: dslash_batch_table_kernel<kL64><<<grid, kBatchChunk, 0, st>>>(tab, head); break;
+    case LQCD_FP64:
+      if (digits) dslash_batch_table_kernel<kL64><<<grid, kBatchChunk, 0, st>>>(tab, head);
+      else dslash_batch_table_kernel<kL64N><<<grid, kBatchChunk, 0, st>>>(tab, head);
+      break;
     case LQCD_FP32_R12: dslash_batch_table_kernel<kL12><<<grid, kBatchChunk, 0, st>>>(tab, head); break;
     case LQCD_FP32_R8: dslash_batch_table_kernel<kL8><<<grid, kBatchChunk, 0, st>>>(tab, head); break;
     case LQCD_FP32_L16: dslash_batch_table_kernel<kL16><<<grid, kBatchChunk, 0, st>>>(tab, head); break;
@@ -678,12 +690,13 @@ static cudaError_t launch_lf(const Geom& g, const KArgs& k, Epi epi, int tps, in
 // FP64 blocks: one per group of sites, at most one resident wave (the blocks then take several groups each)
 static int fp64_blocks(const Geom& g) { return std::min((g.vh + kFixSites - 1) / kFixSites, kFixResident * kSMs); }
 
+template <bool DIGITS>
 static cudaError_t launch_fp64(const Geom& g, const KArgs& k, Epi epi, cudaStream_t st, bool pdl) {
   const dim3 nb((unsigned)fp64_blocks(g)), bs(kFixThreads);
   switch (epi) {
-    case Epi::Plain: return launch_k(pdl, dslash64_kernel<0>, nb, bs, st, g, k);
-    case Epi::AApply: return launch_k(pdl, dslash64_kernel<1>, nb, bs, st, g, k);
-    default: return launch_k(pdl, dslash64_kernel<2>, nb, bs, st, g, k);
+    case Epi::Plain: return launch_k(pdl, dslash64_kernel<0, DIGITS>, nb, bs, st, g, k);
+    case Epi::AApply: return launch_k(pdl, dslash64_kernel<1, DIGITS>, nb, bs, st, g, k);
+    default: return launch_k(pdl, dslash64_kernel<2, DIGITS>, nb, bs, st, g, k);
   }
 }
 
@@ -731,7 +744,7 @@ cudaError_t launch_dslash(const Geom& g, const GaugeCopies& gc, const DslashArgs
     case LQCD_FP64:
       k.links = gc.ufix;
       k.links64 = gc.u64;
-      return launch_fp64(g, k, a.epi, st, a.pdl);
+      return gc.ufix ? launch_fp64<true>(g, k, a.epi, st, a.pdl) : launch_fp64<false>(g, k, a.epi, st, a.pdl);
     case LQCD_FP32_R12: k.links = gc.u12; return launch_lf<kL12>(g, k, a.epi, tps, bs, st, a.pdl);
     case LQCD_FP32_R8: k.links = gc.u8; return launch_lf<kL8>(g, k, a.epi, tps, bs, st, a.pdl);
     case LQCD_FP32_L16: k.links = gc.u16; return launch_lf<kL16>(g, k, a.epi, tps, bs, st, a.pdl);

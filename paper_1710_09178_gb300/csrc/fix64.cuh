@@ -27,12 +27,55 @@ __device__ __forceinline__ size_t fix_entry(int p, int mu, int i, int vh) {
   return (size_t)(p * 4 + mu) * fix_block_entries(vh) + (size_t)((unsigned)i >> 5) * (9 * 32) + (i & 31);
 }
 
-__device__ __forceinline__ FixLink load_link_fix(const int4* __restrict__ U, int p, int mu, int i, int vh,
-                                                 uint64_t pol) {
-  const int4* b = U + fix_entry(p, mu, i, vh);
+// The links of a field: their digits, or (null: not kept, GaugeCopies) the FP64 copy, which then gives them while they
+// are read: the same digits, so the same results.  The FP64 copy [2][4][9][Vh] is followed by one byte per link, [2][4][Vh]:
+// whether it is within the format.
+struct FixField {
+  const int4* digits;
+  const double2* u64;
+};
+__host__ __device__ __forceinline__ const unsigned char* fix_fits(const double2* u64, int vh) {
+  return reinterpret_cast<const unsigned char*>(u64 + 72 * (size_t)vh);
+}
+
+// A link as it is loaded: its digits, or (DIGITS false) its FP64 entries, with fits from that copy.
+template <bool DIGITS>
+struct FixRaw {
+  int4 e[9];
+  int fits;
+};
+
+template <bool DIGITS>
+__device__ __forceinline__ FixRaw<DIGITS> load_link_fix(const FixField& f, int p, int mu, int i, int vh, uint64_t pol) {
+  FixRaw<DIGITS> r;
+  if constexpr (DIGITS) {
+    const int4* b = f.digits + fix_entry(p, mu, i, vh);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) r.e[j] = ld_stream(b + j * 32, pol);
+  } else {
+    const int4* b = reinterpret_cast<const int4*>(f.u64) + (size_t)(p * 4 + mu) * 9 * vh + i;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) r.e[j] = ld_stream(b + (size_t)j * vh, pol);
+    r.fits = fix_fits(f.u64, vh)[(size_t)(p * 4 + mu) * vh + i];
+  }
+  return r;
+}
+
+// The digits of a loaded link; entry (0, 0) marked where it is outside the format.
+template <bool DIGITS>
+__device__ __forceinline__ FixLink fix_digits(const FixRaw<DIGITS>& r) {
   FixLink L;
 #pragma unroll
-  for (int j = 0; j < 9; ++j) L.e[j] = ld_stream(b + j * 32, pol);
+  for (int j = 0; j < 9; ++j) {
+    if constexpr (DIGITS) {
+      L.e[j] = r.e[j];
+    } else {
+      const Fix2 re = fix_link_entry(__hiloint2double(r.e[j].y, r.e[j].x)), im = fix_link_entry(__hiloint2double(r.e[j].w, r.e[j].z));
+      L.e[j] = make_int4(re.h, re.l, im.h, im.l);
+    }
+  }
+  if constexpr (!DIGITS)
+    if (!r.fits) L.e[0].x = kFixBadLink;
   return L;
 }
 
@@ -90,31 +133,29 @@ struct FixShared {
   int word[4][kFixSites];
 };
 
+template <bool DIGITS>
 struct FixGroup {
   int jf, jb;
-  FixLink Lf;
+  FixRaw<DIGITS> Wf;
 
-  // neighbours, and the forward link's loads: nothing that an earlier kernel of the stream writes.  U null (no
-  // room for the digits): every site is computed in FP64.
-  __device__ __forceinline__ void start(const Geom& g, const int4* U, int p, int i, int mu, uint64_t pol) {
-    if (!U) return;
+  // neighbours, and the forward link's loads: nothing that an earlier kernel of the stream writes
+  __device__ __forceinline__ void start(const Geom& g, const FixField& U, int p, int i, int mu, uint64_t pol) {
     const Site s = site_of(g, p, i);
     jf = neighbour_half(g, neighbour_fwd(g, s, mu));
     jb = neighbour_half(g, neighbour_bwd(g, s, mu));
-    Lf = load_link_fix(U, p, mu, i, g.vh, pol);
+    Wf = load_link_fix<DIGITS>(U, p, mu, i, g.vh, pol);
   }
 
   // The thread's two hops, left in sh.part.  All threads of the block call; a barrier has to follow.
-  __device__ __forceinline__ void hops(FixShared& sh, const Geom& g, const int4* U, const double2* in, int p, int mu,
+  __device__ __forceinline__ void hops(FixShared& sh, const Geom& g, const FixField& U, const double2* in, int p, int mu,
                                        int ls, bool valid, uint64_t pol) const {
-    if (!U) return;  // uniform
     const int vh = g.vh;
     Vec3<double> vf, vb;
-    FixLink Lb;
+    FixRaw<DIGITS> Wb;
     if (valid) {
       vf = ldg_vec(in, jf, vh);
       vb = ldg_vec(in, jb, vh);
-      Lb = load_link_fix(U, 1 - p, mu, jb, vh, pol);
+      Wb = load_link_fix<DIGITS>(U, 1 - p, mu, jb, vh, pol);
       const double w[12] = {vf.c[0].re, vf.c[0].im, vf.c[1].re, vf.c[1].im, vf.c[2].re, vf.c[2].im,
                             vb.c[0].re, vb.c[0].im, vb.c[1].re, vb.c[1].im, vb.c[2].re, vb.c[2].im};
       sh.word[mu][ls] = fix_max_word(w);
@@ -128,9 +169,11 @@ struct FixGroup {
       s.rh[c] = s.ih[c] = 0;
       s.rx[c] = s.ix[c] = 1 << (kFixLow - 1);  // rounds the shift below
     }
+    const FixLink Lf = fix_digits(Wf);
     fix_hop<true>(s, Lf, vf, E);
 #pragma unroll
     for (int c = 0; c < 3; ++c) sh.fwd[mu][c][ls] = make_int2(fix_upper(s.rh[c]), fix_upper(s.ih[c]));
+    const FixLink Lb = fix_digits(Wb);
     fix_hop<false>(s, Lb, vb, E);
     const bool bad = Lf.e[0].x == kFixBadLink || Lb.e[0].x == kFixBadLink;
 #pragma unroll
@@ -146,30 +189,26 @@ struct FixGroup {
   }
 
   // after the barrier: colour c of (D in)(x), c = 0 .. 2
-  static __device__ __forceinline__ Cplx<double> colour(const FixShared& sh, const Geom& g, const int4* U, const double2* U64,
-                                                        const double2* in, int p, int i, int c, int ls) {
-    int E = -1;
+  static __device__ __forceinline__ Cplx<double> colour(const FixShared& sh, const Geom& g, const double2* U64, const double2* in,
+                                                        int p, int i, int c, int ls) {
+    const int w[4] = {sh.word[0][ls], sh.word[1][ls], sh.word[2][ls], sh.word[3][ls]};
+    const int E = fix_block_exponent(w);
     int64_t re = 0, im = 0;
-    bool ok = false;
-    if (U) {
-      const int w[4] = {sh.word[0][ls], sh.word[1][ls], sh.word[2][ls], sh.word[3][ls]};
-      E = fix_block_exponent(w);
-      ok = E >= 0;
-      uint32_t hr = 0, hi = 0;
+    bool ok = E >= 0;
+    uint32_t hr = 0, hi = 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const longlong2 u = sh.part[q][c][ls];
-        const int2 f = sh.fwd[q][c][ls];
-        ok = ok && u.x != kFixBadSum;
-        re += u.x;
-        im += u.y;
-        hr += fix_hop_words(f.x, fix_upper(u.x));
-        hi += fix_hop_words(f.y, fix_upper(u.y));
-      }
-      const bool zero = (w[0] | w[1] | w[2] | w[3]) == 0;  // all neighbours
-      const uint32_t need = fix_needed(w, E);
-      ok = ok && (zero || (hr >= need && hi >= need));
+    for (int q = 0; q < 4; ++q) {
+      const longlong2 u = sh.part[q][c][ls];
+      const int2 f = sh.fwd[q][c][ls];
+      ok = ok && u.x != kFixBadSum;
+      re += u.x;
+      im += u.y;
+      hr += fix_hop_words(f.x, fix_upper(u.x));
+      hi += fix_hop_words(f.y, fix_upper(u.y));
     }
+    const bool zero = (w[0] | w[1] | w[2] | w[3]) == 0;  // all neighbours
+    const uint32_t need = fix_needed(w, E);
+    ok = ok && (zero || (hr >= need && hi >= need));
     if (!ok) {
       const Vec3<double> d = site64_fma(g, U64, in, p, i);
       return c == 0 ? d.c[0] : c == 1 ? d.c[1] : d.c[2];

@@ -88,8 +88,8 @@ struct SolverDev {
 
 struct GaugeCopies {
   void* block = nullptr;   // the allocation that holds the copies
-  double2* u64 = nullptr;  // [2][4][9][Vh] double2, 1/2 eta*bc folded in
-  int4* ufix = nullptr;    // the digits of u64 (fix64.cuh), null where there is no room for them
+  double2* u64 = nullptr;  // [2][4][9][Vh] double2, 1/2 eta*bc folded in; then a byte per link (FixField)
+  int4* ufix = nullptr;    // the digits of u64 (fix64.cuh), or null: the same results without them, slower
   float* u32 = nullptr;    // [2][4][18][Vh] floats (float4 x4 + float2), 1/2 eta*bc folded in
   float4* u12 = nullptr;   // [2][4][3][Vh] float4, rows 0-1, no sign
   float4* u8 = nullptr;    // [2][4][2][Vh] float4, 8-real form, no sign
@@ -123,6 +123,7 @@ struct lqcd_ctx {
   int df_resid = 1;        // mixed modes: residuals in double-FP32 instead of FP64
   int dslash_tps = 0;
   int dslash_bs = 0;     // FP32 Dslash threads per block (64 or 128; 0 = 128)
+  int fp64_digits = 1;   // keep the digits of the FP64 links where there is room (set_gauge)
   int dslash_order = 0;  // FP32 Dslash block-to-site order (0 linear, 1 halves interleaved)
   lqcd::Workspace* ws = nullptr;
   lqcd::Workspace* ws_extra[lqcd::kMaxRhs - 1] = {};  // systems 1 .. of multi-RHS solves (mshift_cg_multi)
@@ -203,7 +204,7 @@ constexpr int kBatchPerLaunch = 32;
 struct BatchLattice {
   Geom g;
   const void* links;  // the link copy of the batch's precision
-  const double2* links64;  // FP64: the copy behind the fixed-point one
+  const double2* links64;  // FP64 (links: its digits or null, FixField)
   const void* in;
   void* out;
   int out_parity;
@@ -220,7 +221,7 @@ struct BatchTable {
 };
 int batch_items(int vh);
 cudaError_t launch_dslash_batch(const BatchArgs& a, int prec, unsigned* head, int n_sm, cudaStream_t st);
-cudaError_t launch_dslash_batch_table(const BatchTable* dev_table, int n_items, int prec, unsigned* head, int n_sm,
+cudaError_t launch_dslash_batch_table(const BatchTable* dev_table, int n_items, int prec, bool digits, unsigned* head, int n_sm,
                                       cudaStream_t st);
 int dslash_grid_blocks(const Geom& g, int prec, int tps, int bs = 0);
 

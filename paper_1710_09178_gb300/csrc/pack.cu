@@ -45,25 +45,26 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
   for (int j = 0; j < 9; ++j) e[j] = src[j];
   if (u64) {
     double2* b = u64 + (size_t)(p * 4 + mu) * 9 * vh + i;
-#pragma unroll
-    for (int j = 0; j < 9; ++j) b[(size_t)j * vh] = make_double2(half_sign * e[j].x, half_sign * e[j].y);
-  }
-  if (ufix) {
-    int4* b = ufix + fix_entry(p, mu, i, vh);
     double2 u[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) u[j] = make_double2(half_sign * e[j].x, half_sign * e[j].y);
     const bool fits = fix_link_fits(u);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) {
-      int4 w = make_int4(0, 0, 0, 0);
-      if (fits) {
-        const Fix2 re = fix_link_entry(u[j].x), im = fix_link_entry(u[j].y);
-        w = make_int4(re.h, re.l, im.h, im.l);
-      } else if (j == 0) {
-        w.x = kFixBadLink;
+    for (int j = 0; j < 9; ++j) b[(size_t)j * vh] = u[j];
+    const_cast<unsigned char*>(fix_fits(u64, vh))[(size_t)(p * 4 + mu) * vh + i] = fits;
+    if (ufix) {
+      int4* f = ufix + fix_entry(p, mu, i, vh);
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        int4 w = make_int4(0, 0, 0, 0);
+        if (fits) {
+          const Fix2 re = fix_link_entry(u[j].x), im = fix_link_entry(u[j].y);
+          w = make_int4(re.h, re.l, im.h, im.l);
+        } else if (j == 0) {
+          w.x = kFixBadLink;
+        }
+        f[j * 32] = w;
       }
-      b[j * 32] = w;
     }
   }
   if (u32) {

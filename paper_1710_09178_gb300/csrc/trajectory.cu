@@ -285,10 +285,10 @@ __device__ __forceinline__ bool force_accurate(const FixLink& U, const ForceMag&
 // F[l][mu][a] += beta-scaled gauge force components tr(lambda^a F_g); block: 32 sites of one parity, one direction
 // per warp.  The 13 matrix products of a link in FP64 take 1404 multiply-adds, 702 clocks of the SM's FP64 pipe; in
 // fixed point 4212 integer ones, 66 clocks, and about as much again for digits and addresses: 24^3 x 6 (331 776
-// links) 1865 -> 320 us.  Links outside the format, or no digits (Ufix null): FP64.
-__global__ void __launch_bounds__(kForceThreads, 2) gauge_force_kernel(Geom g, const double2* __restrict__ U,
-                                                                       const int4* __restrict__ Ufix, double beta,
-                                                                       double* __restrict__ F) {
+// links) 1865 -> 320 us.  Links outside the format: FP64.  DIGITS: whether the field keeps its digits (FixField).
+template <bool DIGITS>
+__global__ void __launch_bounds__(kForceThreads, 2) gauge_force_kernel(Geom g, const double2* __restrict__ U, FixField Ufix,
+                                                                       double beta, double* __restrict__ F) {
   __shared__ ForceMag mag;  // each thread's own column
   const int vh = g.vh;
   const int nb = (vh + 31) / 32;
@@ -297,13 +297,13 @@ __global__ void __launch_bounds__(kForceThreads, 2) gauge_force_kernel(Geom g, c
   if (i >= vh) return;
   const Site s = site_of(g, p, i);
   double Wre[9], Wim[9];
-  bool ok = Ufix != nullptr;
-  if (ok) {
+  bool ok = true;
+  {
     const uint64_t pol = policy_evict_last();  // every link is read by the 18 staples it is in
     const int xpmu = neighbour_addr(g, neighbour_fwd(g, s, mu));
     const Site sp = site_at(g, xpmu);
     auto link = [&](int parity, int dir, int l) {
-      const FixLink L = load_link_fix(Ufix, parity, dir, l >> 1, vh, pol);
+      const FixLink L = fix_digits(load_link_fix<DIGITS>(Ufix, parity, dir, l >> 1, vh, pol));
       ok = ok && L.e[0].x != kFixBadLink;
       return L;
     };
@@ -593,7 +593,10 @@ extern "C" int rhmc_trajectory(lqcd_ctx* ctx, const lqcd_rhmc_params* prm, doubl
                           prm->prec, &sst);
     if (r != LQCD_OK) return r;
     count(sst);
-    gauge_force_kernel<<<2 * ((g.vh + 31) / 32), 128, 0, st>>>(g, tw->U, ctx->gauge.ufix, prm->beta, tw->F);
+    const FixField links{ctx->gauge.ufix, ctx->gauge.u64};
+    const unsigned nbf = 2 * ((g.vh + 31) / 32);
+    if (links.digits) gauge_force_kernel<true><<<nbf, kForceThreads, 0, st>>>(g, tw->U, links, prm->beta, tw->F);
+    else gauge_force_kernel<false><<<nbf, kForceThreads, 0, st>>>(g, tw->U, links, prm->beta, tw->F);
     nl += 1;
     TJ_CUDA(cudaGetLastError());
     return LQCD_OK;
