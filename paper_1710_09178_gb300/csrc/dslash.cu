@@ -423,8 +423,9 @@ __global__ void __launch_bounds__(kFixThreads, kFixResident) dslash64_kernel(Geo
     grp.hops(sh, g, U, in, p, mu, ls, valid, pol);
     if (i + step < vh) grp.start(g, U, p, i + step, mu, pol);
     __syncthreads();
+    Cplx<double> d;
+    if (mu < 3) d = FixGroup<DIGITS>::colour(sh, g, k.links64, in, p, i, mu, ls, valid);
     if (mine) {
-      const Cplx<double> d = FixGroup<DIGITS>::colour(sh, g, k.links64, in, p, i, mu, ls);
       double2 w = make_double2(d.re, d.im);
       if constexpr (EPI != (int)Epi::Plain) {
         w = make_double2(a * ps.x - d.re, a * ps.y - d.im);
@@ -556,8 +557,9 @@ __device__ __forceinline__ void batch_loop(const BatchLattice* lat, const int* c
         if (valid) grp.start(L.g, U, p, i, mu, pol);
         grp.hops(sh, L.g, U, in, p, mu, ls, valid, pol);
         __syncthreads();
+        Cplx<double> d;
+        if (mu < 3) d = Group::colour(sh, L.g, L.links64, in, p, i, mu, ls, valid);
         if (valid && mu < 3) {
-          const Cplx<double> d = Group::colour(sh, L.g, L.links64, in, p, i, mu, ls);
           static_cast<double2*>(L.out)[(size_t)mu * vh + i] = make_double2(d.re, d.im);
         }
         __syncthreads();

@@ -2,11 +2,15 @@
 //
 // Measured on GB300, half Dslash per graph launch (caches as the previous launches leave them), with FP64
 // multiply-adds and one thread per site before:
-//     8^4 12.0 -> 3.1 us, 16^3x8 12.8 -> 6.7, 24^3x6 30.8 -> 13.1, 32^3x8 69.8 -> 35.4, 48^3x12 329 -> 171
+//     8^4 12.0 -> 3.2 us, 16^3x8 12.8 -> 6.8, 24^3x6 30.8 -> 13.2, 32^3x8 69.8 -> 35.4, 48^3x12 329 -> 166
 // (32^3x8: 163.6 MB, 24 us at the measured HBM rate).  It runs 17.4 M warp instructions there, 45 % of them
 // on the ALU (digits, addresses) and 39 % on the integer multiplier: issue and load latency share the bound.
-// One direction (two hops) per thread, 3 blocks of 128 threads per SM (168 registers): 4 blocks spill and take
-// 39 us, one hop per thread 36.5 us, one thread per site 68.6 us.
+// One direction (two hops) per thread, 3 blocks of 128 threads per SM (168 registers; up to 24 bytes spilled, 132 in the
+// kernels without digits): 4 blocks (128 registers) take 39 us, one hop per thread 36.5 us, one thread per site 68.6 us.
+// Links outside the format throughout (SU(3) times 1.2), computed in FP64 after a look at the digits: 32^3x8 260 -> 110 us,
+// 16^3x8 48 -> 20, since each of a site's three threads computes its own colour only and skips the integer products; 80 us
+// of that is the FP64 pipe (336 multiply-adds per site at 2 per clock and SM).  Deciding it at the first barrier, with
+// all four threads of a site sharing the work, takes 89 us, but costs ordinary links 2 us.
 #pragma once
 
 #include "common.cuh"
@@ -102,22 +106,56 @@ __device__ __forceinline__ void fix_hop(FixAcc& s, const FixLink& L, const Vec3<
   }
 }
 
-// The same site in FP64, for what the format does not take: fma chains per hop, forward minus backward,
-// directions in order.
-static __device__ __noinline__ Vec3<double> site64_fma(Geom g, const double2* __restrict__ U,
-                                                        const double2* __restrict__ in, int p, int i) {
-  const int vh = g.vh;
-  const Site s = site_of(g, p, i);
+// In FP64, for what the format does not take: colour c of hop h of site i (h: direction h / 2, forward or backward), a chain
+// of multiply-adds that reads the row (column) of the link it needs.  The colour is the sum over the directions, in order, of
+// forward minus backward.
+static __device__ __forceinline__ Cplx<double> hop64(const Geom& g, const Site& s, const double2* U, const double2* in, int p,
+                                                      int i, int c, int h) {
+  const int vh = g.vh, mu = h >> 1;
+  const bool fwd = (h & 1) == 0;
+  const int j = neighbour_half(g, fwd ? neighbour_fwd(g, s, mu) : neighbour_bwd(g, s, mu));
+  const double2* u = U + ((size_t)((fwd ? p : 1 - p) * 4 + mu) * 9 + (fwd ? 3 * c : c)) * vh + (fwd ? i : j);
+  const size_t step = (size_t)(fwd ? 1 : 3) * vh;
   const uint64_t pol = policy_evict_first();
-  Vec3<double> d = vzero<double>();
-#pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) {
-    const int jf = neighbour_half(g, neighbour_fwd(g, s, mu)), jb = neighbour_half(g, neighbour_bwd(g, s, mu));
-    Vec3<double> f = vzero<double>(), b = vzero<double>();
-    mv_acc(f, load_link64(U, p, mu, i, vh, pol), ldg_vec(in, jf, vh));
-    mdv_acc(b, load_link64(U, 1 - p, mu, jb, vh, pol), ldg_vec(in, jb, vh));
+  Cplx<double> d = cmake(0.0, 0.0);
+  double2 l[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) d.c[c] = cmake(d.c[c].re + (f.c[c].re - b.c[c].re), d.c[c].im + (f.c[c].im - b.c[c].im));
+  for (int b = 0; b < 3; ++b) l[b] = ld_stream(u + b * step, pol);
+  const Vec3<double> v = ldg_vec(in, j, vh);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) cmac(d, cmake(l[b].x, fwd ? l[b].y : -l[b].y), v.c[b]);
+  return d;
+}
+
+// Colour c of site i for the lanes with want.  All lanes of the warp call.  A few sites (rough fields: one in 300 000): eight
+// lanes take a site's hops side by side; more: each lane its own site.  The same operations, the same bits.
+static __device__ __noinline__ Cplx<double> site64_fma(Geom g, const double2* __restrict__ U, const double2* __restrict__ in,
+                                                        int p, int i, int c, bool want) {
+  Cplx<double> d = cmake(0.0, 0.0);
+  unsigned todo = __ballot_sync(0xffffffffu, want);
+  const int lane = threadIdx.x & 31;
+  if (__popc(todo) > 4) {
+    if (want) {
+      const Site s = site_of(g, p, i);
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) {
+        const Cplx<double> f = hop64(g, s, U, in, p, i, c, 2 * mu), b = hop64(g, s, U, in, p, i, c, 2 * mu + 1);
+        d = cmake(d.re + (f.re - b.re), d.im + (f.im - b.im));
+      }
+    }
+    return d;
+  }
+  for (; todo; todo &= todo - 1) {
+    const int src = __ffs(todo) - 1, is = __shfl_sync(0xffffffffu, i, src);
+    Cplx<double> t = cmake(0.0, 0.0), r = t;
+    if (lane < 8) t = hop64(g, site_of(g, p, is), U, in, p, is, c, lane);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      const double fr = __shfl_sync(0xffffffffu, t.re, 2 * mu), fi = __shfl_sync(0xffffffffu, t.im, 2 * mu);
+      const double br = __shfl_sync(0xffffffffu, t.re, 2 * mu + 1), bi = __shfl_sync(0xffffffffu, t.im, 2 * mu + 1);
+      r = cmake(r.re + (fr - br), r.im + (fi - bi));
+    }
+    if (lane == src) d = r;
   }
   return d;
 }
@@ -170,11 +208,11 @@ struct FixGroup {
       s.rx[c] = s.ix[c] = 1 << (kFixLow - 1);  // rounds the shift below
     }
     const FixLink Lf = fix_digits(Wf);
-    fix_hop<true>(s, Lf, vf, E);
+    if (Lf.e[0].x != kFixBadLink) fix_hop<true>(s, Lf, vf, E);
 #pragma unroll
     for (int c = 0; c < 3; ++c) sh.fwd[mu][c][ls] = make_int2(fix_upper(s.rh[c]), fix_upper(s.ih[c]));
     const FixLink Lb = fix_digits(Wb);
-    fix_hop<false>(s, Lb, vb, E);
+    if (Lb.e[0].x != kFixBadLink) fix_hop<false>(s, Lb, vb, E);
     const bool bad = Lf.e[0].x == kFixBadLink || Lb.e[0].x == kFixBadLink;
 #pragma unroll
     for (int c = 0; c < 3; ++c)
@@ -188,9 +226,9 @@ struct FixGroup {
     return fix_block_exponent(w);
   }
 
-  // after the barrier: colour c of (D in)(x), c = 0 .. 2
+  // after the barrier: colour c of (D in)(x), c = 0 .. 2.  All lanes of the warp call, with valid for those that have a site.
   static __device__ __forceinline__ Cplx<double> colour(const FixShared& sh, const Geom& g, const double2* U64, const double2* in,
-                                                        int p, int i, int c, int ls) {
+                                                        int p, int i, int c, int ls, bool valid) {
     const int w[4] = {sh.word[0][ls], sh.word[1][ls], sh.word[2][ls], sh.word[3][ls]};
     const int E = fix_block_exponent(w);
     int64_t re = 0, im = 0;
@@ -209,9 +247,9 @@ struct FixGroup {
     const bool zero = (w[0] | w[1] | w[2] | w[3]) == 0;  // all neighbours
     const uint32_t need = fix_needed(w, E);
     ok = ok && (zero || (hr >= need && hi >= need));
-    if (!ok) {
-      const Vec3<double> d = site64_fma(g, U64, in, p, i);
-      return c == 0 ? d.c[0] : c == 1 ? d.c[1] : d.c[2];
+    if (__any_sync(0xffffffffu, valid && !ok)) {
+      const Cplx<double> d = site64_fma(g, U64, in, p, i, c, valid && !ok);
+      if (!ok) return d;
     }
     const double sc = __hiloint2double((E - kFixUnit + 1023) << 20, 0);  // 2^(E - kFixUnit): a normal number
     return cmake((double)(long long)re * sc, (double)(long long)im * sc);
