@@ -48,7 +48,10 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
     double2 u[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) u[j] = make_double2(half_sign * e[j].x, half_sign * e[j].y);
-    const bool fits = fix_link_fits(u);
+    float2 f32[9];  // as the FP32 copy below holds them
+#pragma unroll
+    for (int j = 0; j < 9; ++j) f32[j] = make_float2((float)half_sign * (float)e[j].x, (float)half_sign * (float)e[j].y);
+    const bool fits = fix_link_fits(f32);
 #pragma unroll
     for (int j = 0; j < 9; ++j) b[(size_t)j * vh] = u[j];
     const_cast<unsigned char*>(fix_fits(u64, vh))[(size_t)(p * 4 + mu) * vh + i] = fits;
