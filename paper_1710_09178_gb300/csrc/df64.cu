@@ -5,7 +5,7 @@
 // that certify every shift and give the refinement its right-hand sides (Section 3's FP64
 // treatment of these steps).  On GB300 the FP64 units run at about 1/57 of the FP32 rate: an FP64
 // Dslash takes ~75 us on 32^3 x 8 with FP64 multiply-adds and 35 us with integer ones (fix64.cuh).  Here the
-// same residual is computed with FP32 instructions only, in 24 us:
+// same residual is computed with FP32 instructions only, in 22 us:
 //   - every FP64 number u is held as a pair (hi, lo) = (fl32(u), fl32(u - hi)) (about 48 bits);
 //   - of a product (ah + al)(bh + bl), p = fl32(ah bh) enters the running sum s through Knuth's TwoSum; what
 //     s does not take (TwoSum's error, the product's rounding and the cross terms ah bl + al bh; al bl,
@@ -178,15 +178,16 @@ __device__ __forceinline__ void df_reduce(const DfArgs& k, float ds, float dc) {
 // backward) is one double-FP32 sum, and the four are added in order, whatever TPS, so the bits do not
 // depend on how the directions are spread over threads.
 // The block holds NS = blockDim.x / TPS sites; thread t takes directions t / NS ND .. of site t % NS, ND = 4 / TPS.
-// The four sums meet in shared memory (which with TPS = 1 also keeps them out of the registers that the
-// next links are loaded into), and thread sub finishes colours sub, sub + TPS, ..
+// With TPS = 1 the thread adds each direction to its sum as it goes; kept in 24 KB of shared memory per block until the end,
+// the sums take that from the L1 that the neighbours' vectors hit (32^3x8: 23.8 instead of 22.1 us).  With more
+// threads the four sums meet in shared memory, and thread sub finishes colours sub, sub + TPS, ..
 // UPD: the p update folded in (small lattices, one system): EPI 0 takes r + beta in at every neighbour, beta summed from the
 // r update's partials as the p update kernel does, and runs the beta step in the last block; EPI 1 takes r + beta x at its
 // own site and stores it in x.  The same operations, the same bits.
 template <int EPI, int TPS, bool UPD>
 __global__ void __launch_bounds__(kDfThreads, UPD ? 2 : 4) df_dslash_kernel(Geom g, const __grid_constant__ PerSys<DfArgs> pk) {
   constexpr int NS = kDfThreads / TPS, ND = 4 / TPS;
-  __shared__ float4 part[4][3][NS];
+  __shared__ float4 part[TPS == 1 ? 1 : 4][3][NS];
   const DfArgs& k = pk.s[blockIdx.y];
   const int vh = g.vh;
   const int sub = threadIdx.x / NS, ls = threadIdx.x % NS;
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(kDfThreads, UPD ? 2 : 4) df_dslash_kernel(Geom
       }
   };
   if (TPS > 1) load_own();
+  float4 sum[3];  // TPS = 1: of the directions so far
   if (valid) {
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
@@ -290,7 +292,16 @@ __global__ void __launch_bounds__(kDfThreads, UPD ? 2 : 4) df_dslash_kernel(Geom
         df_hop(sr, cr, si, ci, Uh, Ul, vh3, vl3, fwd);
       }
 #pragma unroll
-      for (int c = 0; c < 3; ++c) part[mu][c][ls] = make_float4(sr[c], cr[c], si[c], ci[c]);
+      for (int c = 0; c < 3; ++c) {
+        if (TPS > 1) {
+          part[mu][c][ls] = make_float4(sr[c], cr[c], si[c], ci[c]);
+        } else if (d == 0) {
+          sum[c] = make_float4(sr[c], cr[c], si[c], ci[c]);
+        } else {
+          df_add(sum[c].x, sum[c].y, sr[c], cr[c]);
+          df_add(sum[c].z, sum[c].w, si[c], ci[c]);
+        }
+      }
     }
   }
   if (TPS > 1) __syncthreads();
@@ -300,12 +311,14 @@ __global__ void __launch_bounds__(kDfThreads, UPD ? 2 : 4) df_dslash_kernel(Geom
   for (int q = 0; q < NC; ++q) {
     const int c = sub + q * TPS;
     if (!valid || c >= 3) continue;
-    float4 t = part[0][c][ls];
+    float4 t = TPS == 1 ? sum[q] : part[0][c][ls];
+    if constexpr (TPS > 1) {
 #pragma unroll
-    for (int mu = 1; mu < 4; ++mu) {
-      const float4 u = part[mu][c][ls];
-      df_add(t.x, t.y, u.x, u.y);
-      df_add(t.z, t.w, u.z, u.w);
+      for (int mu = 1; mu < 4; ++mu) {
+        const float4 u = part[mu][c][ls];
+        df_add(t.x, t.y, u.x, u.y);
+        df_add(t.z, t.w, u.z, u.w);
+      }
     }
     df_finish<EPI>(k, (size_t)c * vh + i, asp, own[q], t.x, t.y, t.z, t.w, ds, dc);
   }
@@ -323,8 +336,8 @@ cudaError_t launch_split_df(const Geom& g, const double2* x, float2* hi, float2*
 // per site (12-operation df_mac): 8^4 6.3 / 3.2 / 2.4, 16^3x8 7.3 / 4.3 / 4.5, 24^3x6 9.8 / 9.5 / 11.2, 32^3x8
 // 24.2 / 25.7 / 30.6, 48^3x12 129 / 132 / 159 (A-applies at 24^3x6 23.5 / 25.9 / 32.4): more threads repeat the
 // site's index arithmetic.  One thread per colour instead gives 4.7, 5.7 and 10.8 us at the first three.
-// With everything here: 8^4 6.2 -> 2.35 us, 16^3x8 7.2 -> 4.05, 24^3x6 9.5 -> 9.8, 32^3x8 23.6 -> 24.5 (A-apply
-// 57.7 -> 56.7), error against quad precision 1.6e-14 -> 7.0e-15 (Gaussian vectors).
+// Against one thread per site and one sum over all directions: 8^4 6.4 -> 2.4 us, 16^3x8 7.4 -> 4.5, 24^3x6 9.5 -> 9.3,
+// 32^3x8 23.0 -> 22.1, 48^3x12 125 -> 124, error against quad precision 1.6e-14 -> 7.0e-15 (Gaussian vectors).
 static int df_tps(const Geom& g) {
   constexpr int kBlocks = 304;
   return g.vh <= kBlocks * kDfThreads / 4 ? 4 : (g.vh <= kBlocks * kDfThreads / 2 ? 2 : 1);
