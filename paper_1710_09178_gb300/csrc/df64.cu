@@ -339,7 +339,7 @@ cudaError_t launch_split_df(const Geom& g, const double2* x, float2* hi, float2*
 // Against one thread per site and one sum over all directions: 8^4 6.4 -> 2.4 us, 16^3x8 7.4 -> 4.5, 24^3x6 9.5 -> 9.3,
 // 32^3x8 23.0 -> 22.1, 48^3x12 125 -> 124, error against quad precision 1.6e-14 -> 7.0e-15 (Gaussian vectors).
 static int df_tps(const Geom& g) {
-  constexpr int kBlocks = 304;
+  constexpr int kBlocks = 2 * kSMs;
   return g.vh <= kBlocks * kDfThreads / 4 ? 4 : (g.vh <= kBlocks * kDfThreads / 2 ? 2 : 1);
 }
 int df_dslash_grid_blocks(const Geom& g) {
@@ -592,14 +592,6 @@ __global__ void __launch_bounds__(kFlushThreads) df_flush_kernel(int n3, const _
   close_window(sd, m, a.ticket);
 }
 
-// (hi, lo) vectors -> FP64 (x = hi + lo, exact), one thread per complex component
-__global__ void __launch_bounds__(256) df_to_fp64_kernel(int n3, const float2* __restrict__ v, double2* __restrict__ x) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= n3) return;
-  const float2 h = v[o], l = v[o + n3];
-  x[o] = make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
-}
-
 cudaError_t launch_df_init(const Geom& g, const double2* b64, void* r, void* p, SolverDev* sd, const InitParams& ip,
                            double* partials, unsigned* ticket, cudaStream_t st) {
   df_init_kernel<<<(g.vh + 255) / 256, 256, 0, st>>>(g, b64, static_cast<float2*>(r), static_cast<float2*>(p), sd, ip,
@@ -619,12 +611,6 @@ cudaError_t launch_df_p_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S,
 cudaError_t launch_df_flush(const Geom& g, const PerSys<DfFlushArgs>& a, int S, cudaStream_t st, bool pdl) {
   const int n3 = 3 * g.vh;
   return launch_k(pdl, df_flush_kernel, flush_grid(n3, S), dim3(kFlushThreads), st, n3, a);
-}
-
-cudaError_t launch_df_to_fp64(const Geom& g, const void* v, double2* x, cudaStream_t st) {
-  const int n3 = 3 * g.vh;
-  df_to_fp64_kernel<<<(n3 + 255) / 256, 256, 0, st>>>(n3, static_cast<const float2*>(v), x);
-  return cudaGetLastError();
 }
 
 }  // namespace lqcd

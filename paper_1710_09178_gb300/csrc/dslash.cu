@@ -26,7 +26,6 @@ namespace lqcd {
 // kL12 and up: signs applied after loading; kL64N: FP64 without digits (FixField)
 enum LinkFmt { kL64N = -1, kL64 = 0, kL32 = 1, kL12 = 2, kL8 = 3, kL16 = 4 };
 
-constexpr int kSMs = 152;         // GB300
 constexpr int kFixResident = 3;  // blocks per SM of the FP64 kernels (168 registers per thread)
 
 struct KArgs {
@@ -131,8 +130,8 @@ __device__ __forceinline__ void dslash_reduce(const KArgs& k, T dsite) {
 }
 
 // Output stage shared by the Dslash kernels: d = (D in)(x) of site i, written as the plain
-// output, the A-apply a * aux - d with Re<aux, out>, or the residual bvec - (a * aux - d) with
-// |out|^2; the sums are reduced over the grid by the last block (every thread of the block calls).
+// output or the A-apply a * aux - d with Re<aux, out>, reduced over the grid by the last block (every thread of the
+// block calls).
 // UPD: the A-apply may have the p update folded in (k.upd_r).
 template <typename T, typename V2, int TPS, int EPI, bool UPD = false>
 __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d, int i, int sub, bool valid,
@@ -156,7 +155,7 @@ __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d
         out[o] = w;
       } else {
         V2 ps = static_cast<const V2*>(k.aux)[o];
-        if constexpr (UPD && EPI == (int)Epi::AApply) {
+        if constexpr (UPD) {
           if (k.upd_r) {  // uniform: p = r + beta p, as the p update kernel forms it
             const T beta = (T)k.sd->beta_f;
             const V2 r = static_cast<const V2*>(k.upd_r)[o];
@@ -167,14 +166,7 @@ __device__ __forceinline__ void dslash_epilogue(const KArgs& k, const Vec3<T>& d
         }
         T qre = aval * ps.x - d.c[c].re;
         T qim = aval * ps.y - d.c[c].im;
-        if constexpr (EPI == (int)Epi::AApply) {
-          dsite += ps.x * qre + ps.y * qim;
-        } else {
-          V2 bv = static_cast<const V2*>(k.bvec)[o];
-          qre = bv.x - qre;
-          qim = bv.y - qim;
-          dsite += qre * qre + qim * qim;
-        }
+        dsite += ps.x * qre + ps.y * qim;
         V2 w;
         w.x = qre;
         w.y = qim;
@@ -657,6 +649,7 @@ cudaError_t launch_dslash_batch_table(const BatchTable* tab, int n_items, int pr
 
 template <int LF, int TPS>
 static cudaError_t launch_tps(const Geom& g, const KArgs& k, Epi epi, cudaStream_t st, int bs, bool pdl) {
+  if (epi == Epi::Resid) return cudaErrorInvalidValue;  // FP64 (launch_fp64) and double-FP32 only
   long long threads = (long long)g.vh * TPS;
   unsigned nb = (unsigned)((threads + bs - 1) / bs);
   // At most one block per SM: all loads at once.  Half Dslash per graph launch, 18-real links: 8^4 2.32 -> 1.98 us, 16^3x8
@@ -665,18 +658,12 @@ static cudaError_t launch_tps(const Geom& g, const KArgs& k, Epi epi, cudaStream
   if constexpr (TPS == 1) {
     if (nb <= kSMs) {
       if (epi == Epi::Plain && k.upd_r) return launch_k(pdl, dslash_pupdate_kernel<LF>, dim3(nb + 1), dim3(128), st, g, k);
-      switch (epi) {
-        case Epi::Plain: return launch_k(pdl, dslash_kernel<LF, 1, 0, true>, dim3(nb), dim3(bs), st, g, k);
-        case Epi::AApply: return launch_k(pdl, dslash_kernel<LF, 1, 1, true>, dim3(nb), dim3(bs), st, g, k);
-        default: return launch_k(pdl, dslash_kernel<LF, 1, 2, true>, dim3(nb), dim3(bs), st, g, k);
-      }
+      if (epi == Epi::Plain) return launch_k(pdl, dslash_kernel<LF, 1, 0, true>, dim3(nb), dim3(bs), st, g, k);
+      return launch_k(pdl, dslash_kernel<LF, 1, 1, true>, dim3(nb), dim3(bs), st, g, k);
     }
   }
-  switch (epi) {
-    case Epi::Plain: return launch_k(pdl, dslash_kernel<LF, TPS, 0>, dim3(nb), dim3(bs), st, g, k);
-    case Epi::AApply: return launch_k(pdl, dslash_kernel<LF, TPS, 1>, dim3(nb), dim3(bs), st, g, k);
-    default: return launch_k(pdl, dslash_kernel<LF, TPS, 2>, dim3(nb), dim3(bs), st, g, k);
-  }
+  if (epi == Epi::Plain) return launch_k(pdl, dslash_kernel<LF, TPS, 0>, dim3(nb), dim3(bs), st, g, k);
+  return launch_k(pdl, dslash_kernel<LF, TPS, 1>, dim3(nb), dim3(bs), st, g, k);
 }
 
 template <int LF>

@@ -13,6 +13,8 @@
 
 namespace lqcd {
 
+constexpr int kSMs = 152;  // GB300
+
 // Device-resident state of one shifted-CG solve (scalars, per-shift recurrences
 // and the coefficients of the pending window of shift-vector updates).
 constexpr int kMaxShifts = LQCD_MAX_SHIFTS;
@@ -290,7 +292,6 @@ cudaError_t launch_df_r_update(const Geom& g, const PerSys<DfUpdArgs>& a, int n,
 cudaError_t launch_df_p_update(const Geom& g, const PerSys<DfUpdArgs>& a, int S, cudaStream_t st, bool pdl);
 int df_dslash_grid_blocks(const Geom& g);  // blocks (= partials) of one double-FP32 Dslash launch
 cudaError_t launch_df_flush(const Geom& g, const PerSys<DfFlushArgs>& a, int S, cudaStream_t st, bool pdl);
-cudaError_t launch_df_to_fp64(const Geom& g, const void* v, double2* x, cudaStream_t st);
 cudaError_t launch_df_to_fp64_many(const Geom& g, void* const* v, double2* const* x, int n, cudaStream_t st);
 
 // solver.cu

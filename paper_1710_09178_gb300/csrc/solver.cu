@@ -556,13 +556,6 @@ __global__ void window_end_kernel(cudaGraphConditionalHandle handle, const __gri
 }
 
 // x += e (FP64 internal vectors)
-__global__ void axpy64_kernel(int n3, double2* __restrict__ x, const double2* __restrict__ e) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n3) return;
-  double2 a = x[i], b = e[i];
-  x[i] = make_double2(a.x + b.x, a.y + b.y);
-}
-
 // An FP32 number as FP64 by integer operations: the conversion instruction runs on the FP64 pipe, 2 lanes per clock and
 // SM.  Exact; zeros, denormals, infinities and NaN take the instruction.
 __device__ __forceinline__ double widen(float f) {
@@ -649,7 +642,7 @@ struct Workspace {
   void* xdf[kMaxShifts] = {};  // the solutions as (hi, lo) FP32 pairs during the solve (xdfmode)
   bool xdfmode = false;        // every mode but LQCD_FP64 (with double-FP32 residuals)
   int pairs = 0;               // the last solve left this many solutions as pairs only (xk is not current)
-  double2 *b64 = nullptr, *r64 = nullptr, *tmp64 = nullptr, *e64 = nullptr, *rb64 = nullptr;
+  double2 *b64 = nullptr, *r64 = nullptr, *tmp64 = nullptr;
   // double-FP32 residuals (mixed modes): x, D_oe x and b as (hi, lo) pairs
   bool df = false;
   float2 *dfx_h = nullptr, *dfx_l = nullptr, *dft_h = nullptr, *dft_l = nullptr, *dfb_h = nullptr, *dfb_l = nullptr;
@@ -697,7 +690,7 @@ static void destroy_workspace(Workspace* w) {
   if (!w) return;
   for (auto& kv : w->graphs) cudaGraphExecDestroy(kv.second);
   void* bufs[] = {w->dfx_h, w->dfx_l, w->dft_h, w->dft_l, w->dfb_h, w->dfb_l,
-                  w->r, w->p, w->q, w->tmp, w->ring, w->b64, w->r64, w->tmp64, w->e64, w->rb64, w->sd,
+                  w->r, w->p, w->q, w->tmp, w->ring, w->b64, w->r64, w->tmp64, w->sd,
                   w->ru_count, w->partials, w->tickets, w->dr, w->dp, w->dq, w->dtmp, w->dring, w->cpartials};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -774,8 +767,6 @@ static int alloc_workspace(lqcd_ctx* ctx, int prec, int n, Workspace** slot, cud
   LQ_CUDA(cudaMalloc(&w->b64, w->dbytes));
   LQ_CUDA(cudaMalloc(&w->r64, w->dbytes));
   LQ_CUDA(cudaMalloc(&w->tmp64, w->dbytes));
-  LQ_CUDA(cudaMalloc(&w->e64, w->dbytes));
-  LQ_CUDA(cudaMalloc(&w->rb64, w->dbytes));
   w->df = prec == LQCD_DF64 || (prec != LQCD_FP64 && ctx->df_resid);
   w->xdfmode = w->df;
   // precision schedule: the mixed modes with double-FP32 residuals start in double-FP32

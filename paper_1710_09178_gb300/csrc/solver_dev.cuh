@@ -250,7 +250,7 @@ constexpr int kFlushThreads = 128;
 // a double-FP32 window); every part loads the window's residuals again (four systems on 8^4: no gain from 3 parts).
 inline dim3 flush_grid(int n3, int S) {
   const int nb = (n3 + kFlushThreads - 1) / kFlushThreads;
-  const int z = 304 / (nb * S);
+  const int z = 2 * kSMs / (nb * S);
   return dim3((unsigned)nb, (unsigned)S, (unsigned)(z < 1 ? 1 : (z > 8 ? 8 : z)));
 }
 
