@@ -32,14 +32,17 @@ __device__ __forceinline__ size_t fix_entry(int p, int mu, int i, int vh) {
 }
 
 // The links of a field: their digits, or (null: not kept, GaugeCopies) the FP64 copy, which then gives them while they
-// are read: the same digits, so the same results.  The FP64 copy [2][4][9][Vh] is followed by one byte per link, [2][4][Vh]:
-// whether it is within the format.
+// are read: the same digits, so the same results.  Behind the copies, which begin with the FP64 one, lies one byte per link,
+// [2][4][Vh]: whether it is within the format.
 struct FixField {
   const int4* digits;
   const double2* u64;
 };
+// bytes of the copies per half-lattice site: FP64, FP32 and its rounding errors, 12-real, 8-real, 16-bit (each a multiple
+// of 256 bytes, Vh being one of 8)
+constexpr size_t kCopyBytes = 8 * (144 + 72 + 72 + 48 + 32 + 24);
 __host__ __device__ __forceinline__ const unsigned char* fix_fits(const double2* u64, int vh) {
-  return reinterpret_cast<const unsigned char*>(u64 + 72 * (size_t)vh);
+  return reinterpret_cast<const unsigned char*>(u64) + kCopyBytes * (size_t)vh;
 }
 
 // A link as it is loaded: its digits, or (DIGITS false) its FP64 entries, with fits from that copy.

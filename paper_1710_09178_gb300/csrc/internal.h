@@ -90,7 +90,7 @@ struct SolverDev {
 
 struct GaugeCopies {
   void* block = nullptr;   // the allocation that holds the copies
-  double2* u64 = nullptr;  // [2][4][9][Vh] double2, 1/2 eta*bc folded in; then a byte per link (FixField)
+  double2* u64 = nullptr;  // [2][4][9][Vh] double2, 1/2 eta*bc folded in; the block begins with it
   int4* ufix = nullptr;    // the digits of u64 (fix64.cuh), or null: the same results without them, slower
   float* u32 = nullptr;    // [2][4][18][Vh] floats (float4 x4 + float2), 1/2 eta*bc folded in
   float4* u12 = nullptr;   // [2][4][3][Vh] float4, rows 0-1, no sign
