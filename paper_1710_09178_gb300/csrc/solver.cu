@@ -555,7 +555,6 @@ __global__ void window_end_kernel(cudaGraphConditionalHandle handle, const __gri
   cudaGraphSetConditional(handle, cont);
 }
 
-// x += e (FP64 internal vectors)
 // An FP32 number as FP64 by integer operations: the conversion instruction runs on the FP64 pipe, 2 lanes per clock and
 // SM.  Exact; zeros, denormals, infinities and NaN take the instruction.
 __device__ __forceinline__ double widen(float f) {

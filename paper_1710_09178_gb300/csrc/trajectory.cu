@@ -285,7 +285,7 @@ __device__ __forceinline__ bool force_accurate(const FixLink& U, const ForceMag&
 // F[l][mu][a] += beta-scaled gauge force components tr(lambda^a F_g); block: 32 sites of one parity, one direction
 // per warp.  The 13 matrix products of a link in FP64 take 1404 multiply-adds, 702 clocks of the SM's FP64 pipe; in
 // fixed point 4212 integer ones, 66 clocks, and about as much again for digits and addresses: 24^3 x 6 (331 776
-// links) 1865 -> 320 us.  Links outside the format: FP64.  DIGITS: whether the field keeps its digits (FixField).
+// links) 1865 -> 335 us, 16 of them for the check (434 without digits).  Links outside the format: FP64.  DIGITS: whether the field keeps its digits (FixField).
 template <bool DIGITS>
 __global__ void __launch_bounds__(kForceThreads, 2) gauge_force_kernel(Geom g, const double2* __restrict__ U, FixField Ufix,
                                                                        double beta, double* __restrict__ F) {
